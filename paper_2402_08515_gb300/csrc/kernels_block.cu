@@ -215,6 +215,23 @@ __device__ __forceinline__ void row_sums_pipe(T (&un)[NH], const T* __restrict__
   }
 }
 
+// The FP64 pipe bounds the FP64 block step (GB300 issues two FP64 operations per clock per
+// SM, all others at 64 times that), so nothing but the FMAs of the sum may go there. -x of a
+// double is an FP64 instruction where it does not fold into its use (a seed that a loop
+// carries), and so is every operand of a select between two sums: the sign is flipped with an
+// integer operation instead, and the optional 2 u_n of the seed is a predicated FMA.
+// 857,375 rows: 63.1 -> 55.3 us per step at 2 columns, 120.0 -> 104.7 us at 4, 207.6 ->
+// 204.9 us at 8 (where the row loads' latency shares the bound).
+__device__ __forceinline__ double neg(double x) {
+  return __hiloint2double(__double2hiint(x) ^ static_cast<int>(0x80000000u), __double2loint(x));
+}
+__device__ __forceinline__ double fma_if(bool p, double a, double b, double c) {
+  asm("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\t@q fma.rn.f64 %0, %1, %2, %0;\n\t}"
+      : "+d"(c)
+      : "d"(a), "d"(b), "r"(static_cast<int>(p)));
+  return c;
+}
+
 // g: the rows the sums gather from (x itself for the leapfrog, the fourth-order stage
 // otherwise); x seeds each row with 2 u_n - u_{n-1}.
 // LPR lanes share a row: LPR = 1 gives a lane a whole row of NB columns and a warp a
@@ -302,7 +319,7 @@ __global__ void __launch_bounds__(256, MINB)
 #pragma unroll
     for (int j = 0; j < NH; ++j) {
       if constexpr (kF32) un[j] = __fsub_rn(__fmul_rn(2.0f, xi[j]), pi[j]);
-      else un[j] = A.fold2 ? -pi[j] : 2.0 * xi[j] - pi[j];  // A.fold2: 2 x_j is in the diagonal
+      else un[j] = fma_if(!A.fold2, 2.0, xi[j], neg(pi[j]));  // A.fold2: 2 x_j is in the diagonal
     }
     if constexpr (PB > 0) {
       if (A.dcol) row_sums_pipe<T, NB, NH, PB>(un, vp, A.dcol + beg + rs, static_cast<int>(row), w, g, co);
@@ -376,14 +393,18 @@ __global__ void __launch_bounds__(256, MINB)
             store_row<NH>(acc_c + at, ac);
           }
         } else {
+          // the accumulator starts at its first term's product: fma(h, u, -0) = h u to the bit
           double na[NH];
-          const int t0 = 3 - nterm;
-          if (!init) load_plain<NH>(acc_s + at, na);
+          if (init) {
+#pragma unroll
+            for (int j = 0; j < NH; ++j) na[j] = -0.0;
+          } else {
+            load_plain<NH>(acc_s + at, na);
+          }
 #pragma unroll 1
-          for (int t = t0; t < 3; ++t) {
+          for (int t = 3 - nterm; t < 3; ++t) {
             double uu[NH];
             term_row(t, uu);
-            const bool fresh = init && t == t0;  // the accumulator starts at its first term's product
             int tb = -1;
             double h = 0.0;
 #pragma unroll
@@ -392,7 +413,7 @@ __global__ void __launch_bounds__(256, MINB)
                 tb = table_of(j);
                 h = ahi[(tf + tb) * Lp1 + step - 1 + t];
               }
-              na[j] = fresh ? h * uu[j] : fma(h, uu[j], na[j]);
+              na[j] = fma(h, uu[j], na[j]);
             }
           }
           if constexpr (LAST) {
