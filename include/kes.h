@@ -76,8 +76,10 @@ typedef struct kes_opts {
   int32_t block_b;     /* largest number of start vectors filtered together (columns of kes_filter_apply and
                           the block size of kes_block_krylov_solve), 1..8; blocks of 2, 4 or 8 columns run
                           as one SpMM step (row-major state), other sizes are padded to the next of them */
-  int32_t autotune;    /* 1: kes_create times every launch shape of the step kernel on this matrix and keeps the
-                          fastest (results do not depend on the choice); 0: use step_variant */
+  int32_t autotune;    /* 1: the staged step kernels where the matrix allows them (every tile of rows gathers from a few
+                          contiguous runs of rows that fit in shared memory; needs compact_cols), else kes_create
+                          times every launch shape of the step kernels on this matrix and keeps the fastest; 0: the
+                          shape step_variant / blk_variant. Results do not depend on the choice */
   int32_t step_variant; /* launch shape used when autotune is 0 (0 .. number of shapes - 1) */
   void* stream;        /* cudaStream_t for every launch; NULL: the context creates its own non-blocking stream */
   /* Optional device allocator (e.g. a framework's caching allocator). Both NULL: cudaMalloc / cudaFree. */
@@ -155,9 +157,10 @@ typedef struct kes_stats {
   double filter_ms;         /* device time of the filter applications (CUDA events on the context stream) */
   double solve_other_ms;    /* device time of orthogonalisation, projection and residuals */
   int64_t bytes_per_step;   /* algorithmic HBM bytes of one fused step (see kes_step_bytes) */
-  int32_t step_variant;     /* launch shape of the step kernel in use */
-  int32_t step_grid;        /* its grid size (blocks of 256 threads) */
-  int32_t blk_variant;      /* launch shape of the block (SpMM) step kernel, -1 for single-vector contexts */
+  int32_t step_variant;     /* launch shape of the step kernel in use, -1: the staged kernels */
+  int32_t step_grid;        /* its grid size in blocks */
+  int32_t blk_variant;      /* launch shape of the block (SpMM) step kernel, -1 for single-vector contexts and the
+                               staged kernels */
   int32_t blk_grid;         /* its grid size */
 } kes_stats;
 

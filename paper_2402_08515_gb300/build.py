@@ -20,9 +20,11 @@ LIB = os.path.join(HERE, "libkes.so")
 SOURCES = [
     "csrc/host_math.cpp",
     "csrc/sell.cpp",
+    "csrc/tiles.cpp",
     "csrc/kernels_step.cu",
     "csrc/kernels_blas.cu",
     "csrc/kernels_block.cu",
+    "csrc/kernels_tile.cu",
     "csrc/kes_api.cu",
     "csrc/solver.cu",
     "csrc/noalloc.cu",

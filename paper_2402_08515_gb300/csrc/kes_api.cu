@@ -78,7 +78,55 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
   const bool ho = c->opts.stepper == KES_STEPPER_LEAPFROG4;
   const int L = c->L, F = c->F;  // L: the tables' length (their stride is L + 1)
   const int64_t stride = c->n_pad * NB;
-  if (x2) {
+  if (c->tiled) {
+    TileStep p;
+    p.type = x2 ? kTileX2 : fp64 ? kTileF64 : kTileF32;
+    p.ts = c->tiles[c->tile_of[p.type][log2_nb(NB)]];
+    p.n_sm = c->cfg.n_sm;
+    p.NB = NB;
+    p.n_values = c->nnz_q;
+    p.val = x2 ? static_cast<const void*>(c->step2) : fp64 ? static_cast<const void*>(c->q64) : c->q32;
+    p.fold2 = (x2 || fp64) && c->fold64;
+    void* start = x2 ? static_cast<void*>(c->U2[2]) : fp64 ? static_cast<void*>(c->stage_in) : c->U32[2];
+    void* U[2];
+    for (int j = 0; j < 2; ++j) U[j] = x2 ? static_cast<void*>(c->U2[j]) : fp64 ? static_cast<void*>(c->U64[j]) : c->U32[j];
+    if (x2)
+      launch_init_x2(c->stream, c->A, NB, c->stage_in, c->U2[2], c->acc_s, c->acc_c, stride, F, c->alpha64, L, cpt);
+    else if (!fp64)
+      launch_init_f32(c->stream, c->A, NB, c->stage_in, c->U32[2], c->acc_s, c->acc_c, stride, F, c->alpha64, L, cpt);
+    p.acc_s = x2 || !fp64 ? static_cast<void*>(c->acc_s) : c->stage_out;
+    p.acc_c = c->acc_c;
+    p.acc64 = c->stage_out;
+    p.acc_stride = stride;
+    p.ahi = x2 || !fp64 ? static_cast<const void*>(c->alpha_hi) : c->alpha64;
+    p.alo = c->alpha_lo;
+    p.F = F;
+    p.L = L;
+    p.cpt = cpt;
+    p.flag = c->d_flag;
+    int next = p.type == kTileF64 ? 0 : 1;  // first weighted term not yet in the accumulators
+    for (int s = 0; s < steps; ++s) {
+      p.x = s == 0 ? start : U[(s - 1) & 1];
+      p.prev = s <= 1 ? start : U[s & 1];
+      p.g = p.x;
+      if (ho) {  // fourth order: the step gathers from v = u_n + A u_n / 12
+        TileStep v = p;
+        v.stage4 = true;
+        v.out = fp64 ? static_cast<void*>(c->V64) : c->V32;
+        v.nterm = 0;
+        launch_tile_step(v, c->stream);
+        p.g = v.out;
+        p.chained = true;
+      }
+      p.out = U[s & 1];
+      p.step = s;
+      p.last = s == steps - 1;
+      p.init = false;
+      p.nterm = acc_plan(s, steps, next, p.init);
+      launch_tile_step(p, c->stream);
+      p.chained = true;
+    }
+  } else if (x2) {
     // FP32 pairs: the FP64 step values (fold64 as for the FP64 steps) split once per filter
     const SellDev A64 = c->step_A64();
     launch_init_x2(c->stream, c->A, NB, c->stage_in, c->U2[2], c->acc_s, c->acc_c, stride, F, c->alpha64, L, cpt);
@@ -155,7 +203,14 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
 void ensure_fp64_state(kes_ctx* c) {
   if (!c->U64[0])
     for (int j = 0; j < 2; ++j) c->U64[j] = c->dzero_n<double>(c->n_pad * c->NBcap);
-  if (!c->step64) {
+  if (c->tiled) {
+    if (!c->q64) {
+      c->q64 = c->dzero_n<double>(c->nnz_q);
+      launch_scale_tiles(c->A, c->slice_rec, c->tile_pat, c->cfg.n_sm, c->stream, c->tau2m64, c->q64, nullptr,
+                         c->fold64);
+      KES_CHECK_LAUNCH();
+    }
+  } else if (!c->step64) {
     c->step64 = c->dzero_n<double>(c->nnz_pad);
     launch_scale_values(c->A, c->cfg, c->stream, c->tau2m64, c->step64, nullptr, nullptr, nullptr, c->fold64);
     KES_CHECK_LAUNCH();
@@ -166,9 +221,10 @@ void ensure_fp64_state(kes_ctx* c) {
 // (again after a filter change rescaled those) and the pair state.
 void ensure_x2_state(kes_ctx* c) {
   ensure_fp64_state(c);
-  if (!c->step2) c->step2 = c->dzero_n<float2>(c->nnz_pad);
+  const int64_t count = c->tiled ? c->nnz_q : c->nnz_pad;
+  if (!c->step2) c->step2 = c->dzero_n<float2>(count);
   if (!c->step2_fresh) {
-    launch_split_values(c->stream, c->nnz_pad, c->step64, c->step2);
+    launch_split_values(c->stream, count, c->tiled ? c->q64 : c->step64, c->step2);
     KES_CHECK_LAUNCH();
     c->step2_fresh = true;
   }
@@ -259,7 +315,7 @@ kes_status check_flag(kes_ctx* c) {
   c->sync();
   if (flag) {
     KES_CUDA(cudaMemsetAsync(c->d_flag, 0, sizeof(int), c->stream));
-    return KES_ERR_UNSTABLE;
+    return flag_status(flag);
   }
   return KES_OK;
 }
@@ -408,6 +464,107 @@ void validate_csr(int64_t n, const int64_t* row_ptr, const int32_t* col, const d
   }
 }
 
+// The step kernels in use, for the statistics: a launch shape, or -1 for the staged ones.
+void shape_stats(kes_ctx* c) {
+  if (c->tiled) {
+    const int type = c->opts.precision == KES_PREC_FP32 ? kTileF32 : kTileF64;
+    c->stats.step_variant = c->stats.blk_variant = -1;
+    c->stats.step_grid = std::min(c->cfg.n_sm, c->tiles[c->tile_of[type][0]].n_tiles);
+    c->stats.blk_grid =
+        c->NBcap > 1 ? std::min(c->cfg.n_sm, c->tiles[c->tile_of[type][log2_nb(c->NBcap)]].n_tiles) : 0;
+    return;
+  }
+  c->stats.step_variant = c->cfg.variant;
+  c->stats.step_grid = c->cfg.grid_step;
+  c->stats.blk_variant = c->NBcap > 1 ? c->cfg.variant_blk : -1;
+  c->stats.blk_grid = c->NBcap > 1 ? c->cfg.grid_blk : 0;
+}
+
+template <typename T>
+T* upload(kes_ctx* c, const std::vector<T>& v) {
+  T* d = c->dalloc_n<T>(static_cast<int64_t>(v.size()));
+  if (!v.empty())
+    KES_CUDA(cudaMemcpyAsync(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, c->stream));
+  return d;
+}
+
+// Lays the matrix out for the staged steps where it allows them: every tile's columns in a few
+// runs of rows, and at least two stages of every precision and block width in shared memory.
+void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, const std::vector<int32_t>& cols,
+                const std::vector<int32_t>& lens) {
+  std::vector<int64_t> row0, rows;
+  for (const MeshInfo& mi : c->meshes) {
+    row0.push_back(mi.row_off);
+    rows.push_back(mi.n_pad);
+  }
+  TileInput in;
+  in.n_slices = n_slices;
+  in.slice_ptr = sp.data();
+  in.col = cols.data();
+  in.len = lens.data();
+  in.n_mesh = c->n_mesh();
+  in.mesh_row0 = row0.data();
+  in.mesh_rows = rows.data();
+  TileLayout lay;
+  if (!build_tile_groups(in, lay)) return;
+  const bool fp32 = c->opts.precision == KES_PREC_FP32, ho = c->opts.stepper == KES_STEPPER_LEAPFROG4;
+  TileHost built[4];
+  bool tried[4] = {}, ok[4] = {};
+  auto tiles_of = [&](int i) {
+    int64_t n = 0;
+    for (int64_t r : rows) n += (r + (kTileGroup >> i) - 1) / (kTileGroup >> i);
+    return n;
+  };
+  for (int type = 0; type < 3; ++type) {
+    if (type != kTileF64 && !fp32) continue;
+    for (int NB = type == kTileX2 ? 2 : 1; NB <= c->NBcap; NB *= 2) {
+      // in order of what the busiest block does, in rows: a tile's own cost counts as 96, and the
+      // first tile has to be there before anything starts
+      int order[4] = {0, 1, 2, 3};
+      auto cost = [&](int i) {
+        return (tiles_of(i) + c->cfg.n_sm - 1) / c->cfg.n_sm * ((kTileGroup >> i) + 96) + (kTileGroup >> i);
+      };
+      std::stable_sort(order, order + 4, [&](int a, int b) { return cost(a) < cost(b); });
+      int pick = -1;
+      for (int want = 4; want >= 2 && pick < 0; want -= 2)
+        for (int q = 0; q < 4 && pick < 0; ++q) {
+          const int i = order[q];
+          if (!tried[i]) {
+            tried[i] = true;
+            ok[i] = build_tiles(in, lay, kTileGroup >> i, built[i]);
+          }
+          if (!ok[i]) continue;
+          const int size = type == kTileF32 ? 4 : 8;
+          if (tile_stages(built[i].R, built[i].max_xrows, built[i].max_w, built[i].max_head, size * NB, size, NB, ho) >=
+              want)
+            pick = i;
+        }
+      if (pick < 0) return;
+      c->tile_of[type][log2_nb(NB)] = pick;
+    }
+  }
+  for (int type = 0; type < 3; ++type)
+    for (int q = 0; q < 4; ++q) {
+      const int i = c->tile_of[type][q];
+      const TileHost& h = built[i];
+      TileSet& ts = c->tiles[i];
+      if (!ok[i] || ts.seg) continue;
+      ts.n_tiles = static_cast<int>(h.seg.size() / (h.max_runs + 2));
+      ts.R = h.R;
+      ts.max_xrows = h.max_xrows;
+      ts.max_w = h.max_w;
+      ts.max_head = h.max_head;
+      ts.max_runs = h.max_runs;
+      ts.seg = upload(c, h.seg);
+      ts.head = upload(c, h.head);
+    }
+  c->slice_rec = upload(c, lay.slice_rec);
+  c->tile_pat = upload(c, lay.pat);
+  c->nnz_q = lay.n_values;
+  c->tiled = true;
+  c->sync();  // the host vectors go out of scope
+}
+
 // Builds the block-diagonal device matrix and the per-row vectors of all meshes.
 void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* row_ptr, const int32_t* const* col,
                    const double* const* val, const double* const* m_diag) {
@@ -447,6 +604,7 @@ void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* r
   std::vector<int32_t> cols(nnz_pad);
   std::vector<double> vals(nnz_pad);
   std::vector<int32_t> smesh(n_slices), rsrc(c->n_pad, -1);
+  std::vector<int32_t> lens(c->n_pad, 0);  // stored entries of each padded row
   std::vector<double> mp(c->n_pad, 0.0), minv(c->n_pad, 0.0);
   bool identity = nm == 1;
   int64_t at = 0;
@@ -466,6 +624,7 @@ void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* r
       const int64_t o = sh.perm.empty() ? i : sh.perm[i];
       rsrc[mi.row_off + i] = static_cast<int32_t>(mi.src_off + o);
       if (mi.row_off + i != mi.src_off + o) identity = false;
+      lens[mi.row_off + i] = static_cast<int32_t>(row_ptr[j][o + 1] - row_ptr[j][o]);
       mp[mi.row_off + i] = m_diag[j][o];
       minv[mi.row_off + i] = 1.0 / m_diag[j][o];
     }
@@ -490,6 +649,7 @@ void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* r
     }
     c->diag_in_rows = diag;
   }
+  if (c->opts.autotune && c->opts.compact_cols) plan_tiles(c, n_slices, sp, cols, lens);
   // compact index for the step kernels: column - row as 16 bits when every entry allows it
   // (padding of a short row points at its own row: difference 0; padding rows past a mesh's
   // last row point at that row)
@@ -524,7 +684,7 @@ void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* r
     int16_t* d_dcol = c->dalloc_n<int16_t>(nnz_pad);
     KES_CUDA(cudaMemcpyAsync(d_dcol, dcol.data(), nnz_pad * sizeof(int16_t), cudaMemcpyHostToDevice, c->stream));
     c->A.dcol = d_dcol;
-    {
+    if (!c->tiled) {
       // pair layout for the single-vector steps: entry k of lane l of slice s at
       // sp2[s] + 64 (k / 2) + 2 l + k % 2, odd widths padded with a zero entry per lane
       std::vector<int64_t> sp2(n_slices + 1, 0);
@@ -611,16 +771,19 @@ kes_status create_impl(kes_ctx** out, int32_t nm, const int64_t* n, const int64_
       KES_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
       c->own_stream = true;
     }
+    c->cfg.n_sm = n_sm;
     build_context(c, nm, n, row_ptr, col, val, m_diag);
     c->fold64 = c->diag_in_rows && c->opts.stepper == KES_STEPPER_LEAPFROG;
     const int64_t np = c->n_pad, nb = c->NBcap;
     c->tau2m64 = c->dzero_n<double>(np);
     if (c->opts.precision == KES_PREC_FP32) {
-      c->step32 = c->dzero_n<float>(c->nnz_pad);
+      if (c->tiled) c->q32 = c->dzero_n<float>(c->nnz_q);  // zero where a row lacks its pattern's entry
+      else c->step32 = c->dzero_n<float>(c->nnz_pad);
       if (c->A.slice_ptr2) c->step32p = c->dzero_n<float>(c->nnz_pair);  // padding stays zero
       for (int j = 0; j < 3; ++j) c->U32[j] = c->dzero_n<float>(np * nb);
     } else {
-      c->step64 = c->dzero_n<double>(c->nnz_pad);
+      if (c->tiled) c->q64 = c->dzero_n<double>(c->nnz_q);
+      else c->step64 = c->dzero_n<double>(c->nnz_pad);
       if (c->A.slice_ptr2 && c->fold64) c->step64p = c->dzero_n<double>(c->nnz_pair);  // padding stays zero
       for (int j = 0; j < 2; ++j) c->U64[j] = c->dzero_n<double>(np * nb);
     }
@@ -637,13 +800,10 @@ kes_status create_impl(kes_ctx** out, int32_t nm, const int64_t* n, const int64_
     c->cfg.variant_blk = c->opts.blk_variant;
     c->cfg.grid_blk =
         n_sm * blk_blocks_per_sm(fp32, c->NBcap > 1 ? c->NBcap : 2, c->opts.blk_variant, c->cfg.block_step);
-    if (c->opts.autotune) tune_steps(c);
+    if (c->opts.autotune && !c->tiled) tune_steps(c);
     c->sync();
     c->stats.bytes_per_step = kes_step_bytes(c, 1, 1);
-    c->stats.step_variant = c->cfg.variant;
-    c->stats.step_grid = c->cfg.grid_step;
-    c->stats.blk_variant = c->NBcap > 1 ? c->cfg.variant_blk : -1;
-    c->stats.blk_grid = c->NBcap > 1 ? c->cfg.grid_blk : 0;
+    shape_stats(c);
     return KES_OK;
   });
   if (st != KES_OK) {
@@ -715,6 +875,9 @@ kes_status set_weights_impl(kes_ctx* c, int32_t F, const double* alpha, const do
     if (c->step64 || c->step32)
       launch_scale_values(c->A, c->cfg, c->stream, c->tau2m64, c->step64, c->step32, c->step64p, c->step32p,
                           c->fold64);
+    if (c->tiled)
+      launch_scale_tiles(c->A, c->slice_rec, c->tile_pat, c->cfg.n_sm, c->stream, c->tau2m64, c->q64, c->q32,
+                         c->fold64);
     c->step2_fresh = false;  // the FP32-pair values follow step64 at their next use
     KES_CHECK_LAUNCH();
     ensure_stage_out(c, F);
@@ -1077,10 +1240,7 @@ kes_status kes_reset_stats(kes_ctx* c) {
     const int64_t bps = c->stats.bytes_per_step;
     c->stats = kes_stats{};
     c->stats.bytes_per_step = bps;
-    c->stats.step_variant = c->cfg.variant;
-    c->stats.step_grid = c->cfg.grid_step;
-    c->stats.blk_variant = c->NBcap > 1 ? c->cfg.variant_blk : -1;
-    c->stats.blk_grid = c->NBcap > 1 ? c->cfg.grid_blk : 0;
+    shape_stats(c);
     return KES_OK;
   });
 }

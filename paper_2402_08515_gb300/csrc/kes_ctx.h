@@ -75,6 +75,10 @@ struct GraphEntry {
   int64_t nodes = 0;
 };
 
+// The status a step kernel's flag stands for: bit 0 non-finite accumulators, bit 1 a wait that
+// ran out.
+inline kes_status flag_status(int flag) { return flag & 2 ? KES_ERR_TIMEOUT : KES_ERR_UNSTABLE; }
+inline int log2_nb(int NB) { return NB >= 8 ? 3 : NB >= 4 ? 2 : NB >= 2 ? 1 : 0; }
 inline int nb_for(int b) { return b <= 1 ? 1 : b <= 2 ? 2 : b <= 4 ? 4 : 8; }
 
 }  // namespace kes
@@ -100,6 +104,17 @@ struct kes_ctx {
   float* step32 = nullptr;        // the same in FP32 (FP32 steps)
   float* step32p = nullptr;       // the FP32 ones in the pair layout (A.slice_ptr2), if built
   int64_t nnz_pair = 0;           // entries of the pair layout (with its padding)
+  // staged steps (kernels_tile.cu), where the matrix allows them and no launch shape was asked
+  // for: the step values in the order of the tiles, one tile set per number of rows in use, and
+  // which of them a precision and block width takes
+  bool tiled = false;
+  double* q64 = nullptr;
+  float* q32 = nullptr;
+  int64_t nnz_q = 0;
+  int4* slice_rec = nullptr;
+  int32_t* tile_pat = nullptr;
+  kes::TileSet tiles[4];          // of 256, 128, 64 and 32 rows
+  int tile_of[3][4] = {};         // [TileType][log2 NB]
   bool diag_in_rows = false;      // every row of the SELL layout stores its diagonal among its slice's
                                   // width (a real entry or padding): the 2 u_n can fold into A
   bool fold64 = false;            // the FP64 step values hold A + 2I (leapfrog and diag_in_rows)

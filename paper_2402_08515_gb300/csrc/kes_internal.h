@@ -65,6 +65,94 @@ struct SellDev {
   const int32_t* slice_mesh = nullptr;
 };
 
+// ---------------------------------------------------------------- staged tiles
+// The matrix as the staged step kernels (kernels_tile.cu) read it. A tile is up to R rows; what
+// its rows gather lies in a few runs of rows, which are copied to shared memory as they are.
+// Rows are grouped by kTileGroup first: a group's slices have one width, and one pattern where
+// their rows are shifted copies of one another (tensor grids): the ascending column - row
+// differences that occur in any of them, entry k of every row at difference k, zero where a row
+// lacks it (kind 0). Other groups store each entry's place among the tile's staged rows in 16
+// bits (kind 1).
+constexpr int kTileGroup = 256;
+constexpr int kMaxRuns = 28;            // runs of a tile: one per lane of the copying warp, four left
+constexpr int kMaxStagedRows = 8192;    // rows a tile may stage (its shared memory is checked on top)
+constexpr int kMaxTileWidth = 1024;
+struct TileInput {
+  int64_t n_slices = 0;
+  const int64_t* slice_ptr = nullptr;
+  const int32_t* col = nullptr;
+  const int32_t* len = nullptr;         // stored entries of each padded row (0 past a mesh's last row)
+  int n_mesh = 0;
+  const int64_t* mesh_row0 = nullptr;
+  const int64_t* mesh_rows = nullptr;   // padded
+};
+struct TileGroup {
+  int64_t row0 = 0, beg = 0;            // beg: first value / 32
+  int rows = 0, mesh = 0, w = 0, kind = 1, pattern = 0;
+};
+struct TileLayout {
+  std::vector<TileGroup> groups;
+  std::vector<std::vector<int32_t>> patterns;
+  std::vector<int4> slice_rec;          // {first value / 32, width, kind, position in pat}
+  std::vector<int32_t> pat;
+  int64_t n_values = 0;
+};
+struct TileHost {
+  int R = 0, max_xrows = 0, max_w = 0, max_head = 0, max_runs = 0;
+  std::vector<int4> seg, head;          // see TileSet
+};
+// Place of entry k of a lane in a slice of width w: quads of entries side by side, then what an
+// odd width leaves as a pair and / or a single.
+int64_t quad_pos(int64_t w, int64_t k, int64_t lane);
+// false: the matrix is not staged (rows too uneven, or columns too scattered)
+bool build_tile_groups(const TileInput& in, TileLayout& out);
+bool build_tiles(const TileInput& in, const TileLayout& lay, int R, TileHost& out);
+
+struct TileSet {
+  int n_tiles = 0, R = 0, max_xrows = 0, max_w = 0, max_head = 0, max_runs = 0;
+  // per tile max_runs + 2: its runs {first row, rows, staged row, 0}, the missing ones empty; its
+  // own rows {first row, rows, 0, 0}; {first value / 32, values, place of its head in 16 bytes, the
+  // head's bytes}
+  const int4* seg = nullptr;
+  // heads: {width, kind, 0, 0}, {first row, rows, mesh, staged row of the first row}, then the
+  // staged row that the first row's entry k lies at (kind 0) or every entry's staged row in 16 bits,
+  // in the order of quad_pos (kind 1)
+  const int4* head = nullptr;
+};
+
+// One staged step (or, stage4, the fourth-order stage) of an NB-column block, as
+// launch_step_f64 / launch_step_blk_* / launch_step_x2 define it; prev = x for the first step.
+enum TileType { kTileF64, kTileF32, kTileX2 };
+struct TileStep {
+  TileType type = kTileF64;
+  TileSet ts;
+  int n_sm = 0, NB = 1;
+  bool stage4 = false;
+  const void* val = nullptr;
+  const void* x = nullptr;
+  const void* g = nullptr;
+  const void* prev = nullptr;
+  void* out = nullptr;
+  void* acc_s = nullptr;
+  void* acc_c = nullptr;
+  double* acc64 = nullptr;
+  int64_t acc_stride = 0;  // n_pad * NB
+  int64_t n_values = 0;
+  const void* ahi = nullptr;
+  const void* alo = nullptr;
+  int F = 1, L = 0, step = 0, cpt = 0, nterm = 0;
+  bool init = false, last = false, fold2 = false;
+  bool chained = false;    // the launch before it in the stream is a staged step of the same filter
+  int* flag = nullptr;
+};
+void launch_tile_step(const TileStep& p, cudaStream_t st);
+// Stages of a tile set's ring that fit a block's shared memory (2 or more: it can run).
+int tile_stages(int R, int max_xrows, int max_w, int max_head, int row_bytes, int value_bytes, int NB, bool ho);
+// Step values in the order of the tiles (q64 / q32, either may be null), see launch_scale_values.
+struct SellDev;
+void launch_scale_tiles(const SellDev& A, const int4* slice_rec, const int32_t* pat, int n_sm, cudaStream_t st,
+                        const double* tau2m, double* q64, float* q32, bool fold2);
+
 struct LaunchCfg {
   int grid_step = 0;   // blocks of the step / SpMV kernels (grid-stride over slices)
   int block_step = 256;

@@ -182,7 +182,7 @@ std::vector<char> BlockSolver::orthogonalise(int jj) {
   c_->sync();
   if (flag) {
     KES_CUDA(cudaMemsetAsync(c_->d_flag, 0, sizeof(int), s_));
-    throw KesError{KES_ERR_UNSTABLE};
+    throw KesError{flag_status(flag)};
   }
   // phase 2 for the vectors that are not dependent: b_k = w / ||w||_M, S b_k (one
   // launch per interval over all meshes), the new column b_i^T S b_k of H
