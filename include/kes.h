@@ -152,8 +152,9 @@ typedef struct kes_result {
 /* Counters accumulated by a context since creation or kes_reset_stats. */
 typedef struct kes_stats {
   int64_t filter_calls;     /* filter applications (one per start-vector block) */
-  int64_t filter_steps;     /* fused leapfrog steps launched (kernel launches of the step kernel) */
-  int64_t kernel_launches;  /* every kernel this library launched (graph nodes counted one by one) */
+  int64_t filter_steps;     /* fused leapfrog steps launched */
+  int64_t kernel_launches;  /* every kernel this library launched; graph nodes, and the steps of a small matrix's
+                               filter that runs as one kernel, counted one by one */
   double filter_ms;         /* device time of the filter applications (CUDA events on the context stream) */
   double solve_other_ms;    /* device time of orthogonalisation, projection and residuals */
   int64_t bytes_per_step;   /* algorithmic HBM bytes of one fused step (see kes_step_bytes) */

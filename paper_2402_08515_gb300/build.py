@@ -25,6 +25,7 @@ SOURCES = [
     "csrc/kernels_blas.cu",
     "csrc/kernels_block.cu",
     "csrc/kernels_tile.cu",
+    "csrc/kernels_resident.cu",
     "csrc/kes_api.cu",
     "csrc/solver.cu",
     "csrc/noalloc.cu",

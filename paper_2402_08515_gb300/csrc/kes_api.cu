@@ -199,6 +199,18 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
   return g_launches - before;
 }
 
+// Whether a filter application runs as one resident kernel: it fits, and a block has few enough
+// stored entries that 16 SMs a column beat a chain of launches over all of them. In FP64 the 16
+// SMs' FP64 pipes set the line (us a step, resident / staged: 3,360 entries a block, 16^3 cells,
+// 1.6 / 2.7; 7,168, 128^2 cells, 2.4 / 2.3; 11,520, 24^3 cells, 3.5 / 2.7). In FP32 shared memory
+// does (11,520: 1.4 / 2.3; 20,640, 29^3 cells: 2.2 / 2.6), but eight columns of that size no
+// longer run at once (3,584, 64^2 cells: 0.8 / 2.4; 11,520: 2.8 / 2.6).
+bool resident_filter(const kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
+  if (x2 || c->opts.stepper != KES_STEPPER_LEAPFROG || !c->resident_range) return false;
+  if (c->resident.entries > (fp64 || NB == 8 ? 7000 : 24000)) return false;
+  return resident_fits(c->resident, fp64, cpt ? 1 : c->F, c->n_mesh(), steps);
+}
+
 // The FP64 step kernels in a context of the FP32 form (used by the FP64 refinement).
 void ensure_fp64_state(kes_ctx* c) {
   if (!c->U64[0])
@@ -249,7 +261,12 @@ void run_filter(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
   }
   cudaEvent_t e0 = c->get_event(), e1 = c->get_event();
   KES_CUDA(cudaEventRecord(e0, c->stream));
-  if (c->opts.use_graph) {
+  if (resident_filter(c, NB, fp64, cpt, steps, x2)) {
+    launch_resident(c->A, c->resident, c->resident_range, fp64, fp64 && c->fold64, c->stream, NB, c->tau2m64,
+                    c->stage_in, c->stage_out, c->F, c->alpha64, c->alpha_hi, c->alpha_lo, c->L, steps, cpt,
+                    c->n_mesh(), c->d_flag);
+    KES_CHECK_LAUNCH();
+  } else if (c->opts.use_graph) {
     if (c->g_F != c->F || c->g_L != c->L) {
       c->drop_graphs();
       c->g_F = c->F;
@@ -565,6 +582,31 @@ void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, co
   c->sync();  // the host vectors go out of scope
 }
 
+// The resident filter's slices, entries and column range per block, where they can fit at all.
+void plan_resident(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, const std::vector<int32_t>& cols) {
+  if (n_slices > 32 * 64 || !resident_available()) return;
+  ResidentPlan p;
+  p.blocks = kResidentBlocks;
+  p.slices = static_cast<int>((n_slices + p.blocks - 1) / p.blocks);
+  std::vector<int2> range(p.blocks, int2{0, 0});
+  for (int b = 0; b < p.blocks; ++b) {
+    const int64_t s0 = std::min<int64_t>(n_slices, int64_t(b) * p.slices), s1 = std::min(n_slices, s0 + p.slices);
+    if (s0 == s1) continue;
+    int32_t lo = static_cast<int32_t>(s0 * kSliceC), hi = static_cast<int32_t>(s1 * kSliceC);
+    for (int64_t e = sp[s0]; e < sp[s1]; ++e) {
+      lo = std::min(lo, cols[e]);
+      hi = std::max(hi, cols[e] + 1);
+    }
+    range[b] = int2{lo, hi};
+    p.xrows = std::max(p.xrows, hi - lo);
+    p.entries = std::max<int>(p.entries, static_cast<int>(sp[s1] - sp[s0]));
+  }
+  if (!resident_fits(p, false, 1, c->n_mesh(), 1)) return;
+  c->resident_range = upload(c, range);
+  c->resident = p;
+  c->sync();
+}
+
 // Builds the block-diagonal device matrix and the per-row vectors of all meshes.
 void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* row_ptr, const int32_t* const* col,
                    const double* const* val, const double* const* m_diag) {
@@ -649,7 +691,10 @@ void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* r
     }
     c->diag_in_rows = diag;
   }
-  if (c->opts.autotune && c->opts.compact_cols) plan_tiles(c, n_slices, sp, cols, lens);
+  if (c->opts.autotune && c->opts.compact_cols) {
+    plan_tiles(c, n_slices, sp, cols, lens);
+    plan_resident(c, n_slices, sp, cols);
+  }
   // compact index for the step kernels: column - row as 16 bits when every entry allows it
   // (padding of a short row points at its own row: difference 0; padding rows past a mesh's
   // last row point at that row)

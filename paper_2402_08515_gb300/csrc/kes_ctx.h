@@ -115,6 +115,10 @@ struct kes_ctx {
   int32_t* tile_pat = nullptr;
   kes::TileSet tiles[4];          // of 256, 128, 64 and 32 rows
   int tile_of[3][4] = {};         // [TileType][log2 NB]
+  // the resident filter (kernels_resident.cu): its plan and the blocks' column ranges, where the
+  // matrix is small enough and no launch shape was asked for
+  kes::ResidentPlan resident;
+  int2* resident_range = nullptr;
   bool diag_in_rows = false;      // every row of the SELL layout stores its diagonal among its slice's
                                   // width (a real entry or padding): the 2 u_n can fold into A
   bool fold64 = false;            // the FP64 step values hold A + 2I (leapfrog and diag_in_rows)

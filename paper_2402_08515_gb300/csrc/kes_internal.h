@@ -153,6 +153,23 @@ struct SellDev;
 void launch_scale_tiles(const SellDev& A, const int4* slice_rec, const int32_t* pat, int n_sm, cudaStream_t st,
                         const double* tau2m, double* q64, float* q32, bool fold2);
 
+// ---------------------------------------------------------------- resident filter
+// A filter application in one kernel by clusters of kResidentBlocks blocks (kernels_resident.cu):
+// every block owns `slices` slices (the last ones fewer); the most stored entries (padding
+// included) and rows of a column range that one of them has.
+constexpr int kResidentBlocks = 16;
+struct ResidentPlan {
+  int blocks = 0, slices = 0, entries = 0, xrows = 0;
+};
+bool resident_available();
+bool resident_fits(const ResidentPlan& p, bool fp64, int tables, int meshes, int steps);
+// r, out: n_pad x NB row-major (out: F of them, one when cpt > 0); the weights as for the steps
+struct SellDev;
+void launch_resident(const SellDev& A, const ResidentPlan& p, const int2* range, bool fp64, bool fold2,
+                     cudaStream_t st, int NB, const double* tau2m, const double* r, double* out, int F,
+                     const double* alpha, const float* ahi, const float* alo, int L, int steps, int cpt, int meshes,
+                     int* flag);
+
 struct LaunchCfg {
   int grid_step = 0;   // blocks of the step / SpMV kernels (grid-stride over slices)
   int block_step = 256;

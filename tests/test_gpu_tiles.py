@@ -93,3 +93,22 @@ def test_scattered_columns_are_not_staged():
     ref, _ = _filter(q, False, 12, 1)
     assert not staged
     np.testing.assert_array_equal(got, ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("b,F,L", [(1, 1, 1), (1, 4, 5), (3, 2, 6), (8, 1, 9)])
+@pytest.mark.parametrize("cells", [(3, 2), (17, 33), (60, 70), (11, 12, 13), (24, 21, 24)])
+def test_resident_filter_equals_the_launch_shapes(cells, b, F, L, precision):
+    """Small matrices run a filter in one kernel (one slice up to the largest that FP64 and eight columns take): same bits."""
+    p = box_grid(cells, extent=tuple(c / 16.0 for c in cells))
+    got, _ = _filter(p, True, L, b, F, precision=precision)
+    ref, _ = _filter(p, False, L, b, F, precision=precision)
+    np.testing.assert_array_equal(got, ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_resident_columns_and_meshes_equal_the_launch_shapes(precision):
+    p = [square_grid(20), box_grid((9, 8, 7)), flared_tube(0.05, length=1.0, r0=0.1, growth=1.0)]
+    got, _ = _filter(p, True, 12, 6, 3, columns=True, precision=precision)
+    ref, _ = _filter(p, False, 12, 6, 3, columns=True, precision=precision)
+    np.testing.assert_array_equal(got, ref)
