@@ -21,8 +21,8 @@
 // less a step at 128^3 cells and 1.0 us at 64^3 (FP32, one column).
 //
 // Microseconds a step, register-staged -> staged (cubes of n^3 cells): one column, 128^3: FP32
-// 36.0 -> 22.7 (the 158 MB an average step cannot do without at 7.0 TB/s), FP64 67.8 -> 62.7 (FP64
-// pipe); 64^3: FP32 6.0 -> 4.5, FP64 11.1 -> 10.2, fourth order 27.6 -> 19.6. FP32, 128^3: 2
+// 36.0 -> 22.7 (the 158 MB an average step cannot do without at 7.0 TB/s), FP64 67.8 -> 59.2 (FP64
+// pipe); 64^3: FP32 6.0 -> 4.5, FP64 11.1 -> 9.9, fourth order 27.6 -> 19.6. FP32, 128^3: 2
 // columns 44.8 -> 30.4, 4 62.3 -> 43.0, 8 84.8 -> 78.6 (shared memory and DRAM). FP64, 96^3: 2
 // columns 55.3 -> 49.9, 4 104.7 -> 94.9, 8 204.9 -> 186.8 (FP64 pipe 97% busy).
 #include <cuda_runtime.h>
@@ -166,8 +166,10 @@ __device__ __forceinline__ void quad(const T* v, int k, int lr, T (&y)[4]) {
   y[3] = b.v[1];
 }
 
-// MODE 0: the step; 1: the stage v = u + A u / 12 of the fourth-order scheme (Remark 2.4).
-template <typename T, int NB, int MODE, int GROUPS>
+// MODE 0: the step; 1: the stage v = u + A u / 12 of the fourth-order scheme (Remark 2.4). FOLD
+// (FP64): the values hold A + 2I; a parameter of the kernel, since a condition in it costs the
+// FP64 pipe one more operation a row (128^3 cells, one column: 62.7 -> 59.2 us a step).
+template <typename T, int NB, int MODE, int GROUPS, bool FOLD>
 __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(const __grid_constant__ TileArgs a) {
   using S = typename std::conditional<std::is_same<T, double>::value, double, float>::type;  // accumulators, weights
   constexpr bool kPair = std::is_same<T, float2>::value, kF64 = std::is_same<T, double>::value;
@@ -336,7 +338,7 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
           }
         } else if constexpr (kF64) {
           un[j].s = neg(pi.v[j]);
-          if (!a.fold2) un[j].s = fma(2.0, xi.v[j], un[j].s);
+          if constexpr (!FOLD) un[j].s = fma(2.0, xi.v[j], un[j].s);
         } else {
           un[j].s = __fsub_rn(__fmul_rn(2.0f, xi.v[j]), pi.v[j]);
         }
@@ -548,13 +550,13 @@ Fit fit_stage(int R, int max_xrows, int max_w, int max_head, int row_bytes, int 
   return f;
 }
 
-template <typename T, int NB, int MODE, int GROUPS>
+template <typename T, int NB, int MODE, int GROUPS, bool FOLD>
 void launch_groups(TileArgs a, int grid, cudaStream_t st) {
   // The stages are a multiple of the groups, so a stage is used by one group and one copying
   // warp of each role only: whoever waits for its next use has seen the last one, and cannot
   // take the phase before that for the one it waits for.
   // the limit is the same for every context: another thread's launch never lowers it
-  cudaFuncSetAttribute(k_tile<T, NB, MODE, GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
+  cudaFuncSetAttribute(k_tile<T, NB, MODE, GROUPS, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
   cudaLaunchConfig_t c{};
   c.gridDim = dim3(grid);
   c.blockDim = dim3(32 * (kGroupWarps + 2) * GROUPS);
@@ -565,15 +567,22 @@ void launch_groups(TileArgs a, int grid, cudaStream_t st) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   c.attrs = at;
   c.numAttrs = a.chained ? 1 : 0;
-  cudaLaunchKernelEx(&c, k_tile<T, NB, MODE, GROUPS>, a);
+  cudaLaunchKernelEx(&c, k_tile<T, NB, MODE, GROUPS, FOLD>, a);
 }
 // Three groups of warps where two stages for each fit, else two (128^3 cells, one column: FP32,
-// six stages, 22.7 us a step with three and 23.8 us with two; FP64, four stages of 45 KB, 62.7 us
-// with two and 78 us with three, which leaves none to be filled while the others are in use).
+// six stages, 22.7 us a step with three and 23.8 us with two; FP64, four stages of 45 KB, 59.2 us
+// with two groups; three (78 us when two took 62.7) leave none to be filled while the others are in use).
 template <typename T, int NB, int MODE>
 void launch_one(const TileArgs& a, int grid, cudaStream_t st) {
-  if (a.stages >= 6) launch_groups<T, NB, MODE, 3>(a, grid, st);
-  else launch_groups<T, NB, MODE, 2>(a, grid, st);
+  if constexpr (std::is_same<T, double>::value && MODE == 0) {
+    if (a.fold2) {
+      if (a.stages >= 6) launch_groups<T, NB, MODE, 3, true>(a, grid, st);
+      else launch_groups<T, NB, MODE, 2, true>(a, grid, st);
+      return;
+    }
+  }
+  if (a.stages >= 6) launch_groups<T, NB, MODE, 3, false>(a, grid, st);
+  else launch_groups<T, NB, MODE, 2, false>(a, grid, st);
 }
 
 template <typename T, int MODE>
