@@ -176,6 +176,8 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
   constexpr int CPL = NB < static_cast<int>(16 / sizeof(T)) ? NB : static_cast<int>(16 / sizeof(T));  // columns per lane
   constexpr int LPR = NB / CPL;           // lanes per row
   constexpr int RPU = kSliceC / LPR;      // rows per warp pass
+  // weight tables' accumulators read ahead, besides the staged first one's, as registers allow
+  constexpr int kAhead = GROUPS == 2 ? 3 : NB <= 2 ? 1 : 0;
   constexpr int kRowBytes = NB * static_cast<int>(sizeof(T));
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[2 * kMaxStages];
@@ -343,6 +345,19 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
           un[j].s = __fsub_rn(__fmul_rn(2.0f, xi.v[j]), pi.v[j]);
         }
       }
+      const int64_t go = static_cast<int64_t>(r1.x) * NB + at;  // this lane's values in a row-major block
+      // the accumulators of more tables than the staged one, read ahead of the row sums (96^3 cells,
+      // 8 columns, 4 tables, FP32 67.5 -> 64.5 us a step; one column, 128^3, 46.5 -> 34.6)
+      Vec<S, CPL> more_s[kAhead + 1], more_c[kAhead + 1];
+      auto load_acc = [&](int f, int64_t go, Vec<S, CPL>& s_, Vec<S, CPL>& c_) {
+        s_ = ld_vec<S, CPL>(static_cast<const S*>(a.acc_s) + f * a.acc_stride + go);
+        if (!kF64) c_ = ld_vec<S, CPL>(static_cast<const S*>(a.acc_c) + f * a.acc_stride + go);
+      };
+      if (accs && nacc > 1) {
+#pragma unroll
+        for (int q = 0; q < kAhead; ++q)
+          if (q + 1 < nacc) load_acc(q + 1, go, more_s[q], more_c[q]);
+      }
       const T* v = vs + (r / kSliceC) * kSliceC * w;
       auto row_at = [&](int row) { return ld_vec<T, CPL>(xs + row * NB + co); };
       auto add = [&](T y, const Vec<T, CPL>& xv) {
@@ -392,7 +407,6 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
         }
         if (rest & 1) add(v[(w - 1) * kSliceC + lr], row_at(q[(w - 1) * kSliceC + lr]));
       }
-      const int64_t go = static_cast<int64_t>(r1.x) * NB + at;  // this lane's values in a row-major block
       Vec<T, CPL> res;
 #pragma unroll
       for (int j = 0; j < CPL; ++j) {
@@ -404,18 +418,11 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
       if constexpr (MODE == 0) {
         // the last nterm of alpha_{n-1} u_{n-1}, alpha_n u_n, alpha_{n+1} u_{n+1}, in that order
         if (a.nterm > 0) {
-          for (int f = 0; f < nacc; ++f) {
+          auto add_terms = [&](int f, Vec<S, CPL>& as, Vec<S, CPL>& ac) {
             const int64_t ga = f * a.acc_stride + go;
-            Vec<S, CPL> as, ac;
             if (kF64 && a.init) {  // it starts at the first term's product: fma(h, u, -0) = h u to the bit
 #pragma unroll
               for (int j = 0; j < CPL; ++j) as.v[j] = static_cast<S>(-0.0);
-            } else if (f == 0) {
-              as = ld_vec<S, CPL>(reinterpret_cast<const S*>(sp + a.off_acc) + at);
-              if (!kF64) ac = ld_vec<S, CPL>(reinterpret_cast<const S*>(sp + a.off_acc) + a.ts.R * NB + at);
-            } else {
-              as = ld_vec<S, CPL>(static_cast<const S*>(a.acc_s) + ga);
-              if (!kF64) ac = ld_vec<S, CPL>(static_cast<const S*>(a.acc_c) + ga);
             }
             auto term = [&](int q, const Vec<T, CPL>& uu) {
 #pragma unroll
@@ -460,10 +467,26 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
               st_vec<S, CPL>(static_cast<S*>(a.acc_s) + ga, as);
               st_vec<S, CPL>(static_cast<S*>(a.acc_c) + ga, ac);
             }
+          };
+          Vec<S, CPL> as, ac;
+          if (accs) {
+            as = ld_vec<S, CPL>(reinterpret_cast<const S*>(sp + a.off_acc) + at);
+            if (!kF64) ac = ld_vec<S, CPL>(reinterpret_cast<const S*>(sp + a.off_acc) + a.ts.R * NB + at);
+          }
+          add_terms(0, as, ac);
+          if (nacc > 1) {
+#pragma unroll
+            for (int q = 0; q < kAhead; ++q)
+              if (q + 1 < nacc) add_terms(q + 1, more_s[q], more_c[q]);
+            for (int f = kAhead + 1; f < nacc; ++f) {
+              load_acc(f, go, as, ac);
+              add_terms(f, as, ac);
+            }
           }
         }
       }
     }
+    // everything read from the stage has been used by now: the copies that follow may overwrite it
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_addr(&bars[kMaxStages + st]));
     st += GROUPS;

@@ -68,6 +68,16 @@ namespace {
 // Largest stable tau * omega of the context's stepper.
 double cfl_bound(const kes_ctx* c) { return c->opts.stepper == KES_STEPPER_LEAPFROG4 ? 2.0 * std::sqrt(3.0) : 2.0; }
 
+// Whether a staged context runs this filter with the register-staged block kernel all the same:
+// eight FP32 columns that each add to several weight tables. The staged step keeps one table's
+// accumulators in its stages; the others' 1 KB a row of 16 is latency that its 16 computing warps
+// do not hide (96^3 cells, us a step: 2 tables 41.6 against 43.9 staged, 4 tables 53.9 against
+// 64.5; with one 35.1 against 33.1, and narrower blocks and FP64 are faster staged with 4, too).
+bool many_tables(const kes_ctx* c, int NB, bool fp64, int cpt, bool x2) {
+  return c->tiled && !fp64 && !x2 && NB == 8 && cpt == 0 && c->F > 1 && c->opts.stepper == KES_STEPPER_LEAPFROG;
+}
+constexpr int kManyTablesShape = 13;  // the shape that the autotuner picks for it on the meshes at hand
+
 // Issues the fused steps of one filter application of an NB-column block on the context
 // stream: stage_in -> stage_out (cpt = 0: F filtered blocks, every column with every
 // weight table; cpt > 0: one block, column j with table min(j / cpt, F - 1)). steps <= L
@@ -78,7 +88,7 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
   const bool ho = c->opts.stepper == KES_STEPPER_LEAPFROG4;
   const int L = c->L, F = c->F;  // L: the tables' length (their stride is L + 1)
   const int64_t stride = c->n_pad * NB;
-  if (c->tiled) {
+  if (c->tiled && !many_tables(c, NB, fp64, cpt, x2)) {
     TileStep p;
     p.type = x2 ? kTileX2 : fp64 ? kTileF64 : kTileF32;
     p.ts = c->tiles[c->tile_of[p.type][log2_nb(NB)]];
@@ -173,6 +183,11 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
     }
   } else {
     const SellDev A32 = c->step_A32();
+    LaunchCfg cfg = c->cfg;
+    if (c->tiled) {
+      cfg.variant_blk = kManyTablesShape;
+      cfg.grid_blk = cfg.n_sm * blk_blocks_per_sm(true, NB, kManyTablesShape, cfg.block_step);
+    }
     launch_init_f32(c->stream, c->A, NB, c->stage_in, c->U32[2], c->acc_s, c->acc_c, stride, F, c->alpha64, L, cpt);
     int next = 1;  // the initialisation added alpha_0 u_0
     for (int s = 0; s < steps; ++s) {
@@ -191,8 +206,8 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
         launch_step_f32(A32, c->cfg, c->stream, first, last, x, g, prev, out, c->acc_s, c->acc_c, c->stage_out,
                         stride, F, c->alpha_hi, c->alpha_lo, L, s, nterm, c->d_flag);
       } else {
-        launch_step_blk_f32(A32, c->cfg, c->stream, NB, first, last, x, g, prev, out, c->acc_s, c->acc_c,
-                            c->stage_out, stride, F, c->alpha_hi, c->alpha_lo, L, s, cpt, nterm, c->d_flag);
+        launch_step_blk_f32(A32, cfg, c->stream, NB, first, last, x, g, prev, out, c->acc_s, c->acc_c, c->stage_out,
+                            stride, F, c->alpha_hi, c->alpha_lo, L, s, cpt, nterm, c->d_flag);
       }
     }
   }
@@ -255,6 +270,11 @@ void run_filter(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
   if (steps <= 0 || steps > c->L) steps = c->L;
   if (x2) ensure_x2_state(c);
   else if (fp64) ensure_fp64_state(c);
+  else if (many_tables(c, NB, fp64, cpt, x2) && !c->step32) {
+    c->step32 = c->dzero_n<float>(c->nnz_pad);  // in the SELL order, kept with the filter from now on
+    launch_scale_values(c->A, c->cfg, c->stream, c->tau2m64, nullptr, c->step32, nullptr, nullptr, false);
+    KES_CHECK_LAUNCH();
+  }
   if (c->opts.stepper == KES_STEPPER_LEAPFROG4) {  // stage buffers before any graph captures them
     if (fp64 && !c->V64) c->V64 = c->dzero_n<double>(c->n_pad * c->NBcap);
     if (!fp64 && !c->V32) c->V32 = c->dzero_n<float>(c->n_pad * c->NBcap);
