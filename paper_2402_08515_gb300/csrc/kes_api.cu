@@ -270,11 +270,6 @@ void run_filter(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
   if (steps <= 0 || steps > c->L) steps = c->L;
   if (x2) ensure_x2_state(c);
   else if (fp64) ensure_fp64_state(c);
-  else if (many_tables(c, NB, fp64, cpt, x2) && !c->step32) {
-    c->step32 = c->dzero_n<float>(c->nnz_pad);  // in the SELL order, kept with the filter from now on
-    launch_scale_values(c->A, c->cfg, c->stream, c->tau2m64, nullptr, c->step32, nullptr, nullptr, false);
-    KES_CHECK_LAUNCH();
-  }
   if (c->opts.stepper == KES_STEPPER_LEAPFROG4) {  // stage buffers before any graph captures them
     if (fp64 && !c->V64) c->V64 = c->dzero_n<double>(c->n_pad * c->NBcap);
     if (!fp64 && !c->V32) c->V32 = c->dzero_n<float>(c->n_pad * c->NBcap);
@@ -936,6 +931,10 @@ kes_status set_weights_impl(kes_ctx* c, int32_t F, const double* alpha, const do
       for (int64_t i = 0; i < mi.n; ++i) t2m[mi.row_off + i] = tau[j] * tau[j] / m[mi.row_off + i];
     }
     KES_CUDA(cudaMemcpyAsync(c->tau2m64, t2m.data(), c->n_pad * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    // the register-staged block kernel's values, where a filter may take it (many_tables)
+    if (c->tiled && !c->step32 && c->opts.precision == KES_PREC_FP32 && c->NBcap == 8 && F > 1 &&
+        c->opts.stepper == KES_STEPPER_LEAPFROG)
+      c->step32 = c->dzero_n<float>(c->nnz_pad);
     // step values A = -tau^2 M^{-1} S (the FP32 ones rounded once from the FP64 product)
     if (c->step64 || c->step32)
       launch_scale_values(c->A, c->cfg, c->stream, c->tau2m64, c->step64, c->step32, c->step64p, c->step32p,
