@@ -40,8 +40,7 @@ if ROOT not in sys.path:
 METRIC = "GDOF*steps/s"
 TTS_TOL = 1e-8
 FALLBACK_HBM_GBS = 6800.0
-STEP_KERNEL_SRC = os.path.join(ROOT, "paper_2402_08515_gb300", "csrc", "kernels_step.cu")
-BLOCK_KERNEL_SRC = os.path.join(ROOT, "paper_2402_08515_gb300", "csrc", "kernels_block.cu")
+STEP_KERNEL_SRC = BLOCK_KERNEL_SRC = os.path.join(ROOT, "paper_2402_08515_gb300", "csrc", "kernels_tile.cu")
 
 
 def parse_args(argv=None):
@@ -203,6 +202,22 @@ def kernel_source_hash(src: str = STEP_KERNEL_SRC) -> str:
         if line:
             code.append(line)
     return hashlib.sha256("\n".join(code).encode()).hexdigest()[:16]
+
+
+def step_bytes(K, h, problems, precision, b, F, L, staged) -> int:
+    """Algorithmic bytes of an average step. The staged kernels read no row pointers, and no columns on tensor grids
+    (rows of a tile are shifted copies of one another) and 2-byte places elsewhere; the launch shapes read what
+    kes_step_bytes counts."""
+    if not staged:
+        return K.kes_step_bytes(h, b, F)
+    n, nnz = sum(p.n for p in problems), sum(p.nnz for p in problems)
+    size = 8 if precision == "fp64" else 4
+    nxt, adds = (0 if size == 8 else 1), 0   # the steps that add weighted terms: every third and the last
+    for s in range(L):
+        if s + 2 - nxt >= 3 or s == L - 1:
+            nxt, adds = s + 2, adds + 1
+    places = 0 if all("extent" in p.meta for p in problems) else 2
+    return (size + places) * nnz + n * b * 3 * size + n * b * 16 * F * adds // L
 
 
 def profiled_traffic(workload: str, src: str = STEP_KERNEL_SRC):
@@ -506,12 +521,12 @@ def batch_filter_measurement(dev, stream, reps: int = 3) -> dict:
                 K.kes_filter_apply(h, R, res, wl.b)
             st = K.kes_get_stats(h)
             step_us = 1e3 * st["filter_ms"] / max(st["filter_steps"], 1)
-            nbytes = K.kes_step_bytes(h, wl.b, F)
+            nbytes = step_bytes(K, h, problems, wl.precision, wl.b, F, wl.L, st["blk_variant"] == -1)
             gbs = nbytes / (step_us / 1e6) / 1e9
             out[f"F{F}"] = {"step_us": step_us, "algorithmic_bytes_per_step": nbytes, "achieved_gbs": gbs,
                             "frac": gbs / peak, "gdof_steps_per_s": n * wl.b / (step_us / 1e6) / 1e9,
                             "finite": bool(torch.isfinite(res).all())}
-        out["kernel"] = "k_step_blk<float,8>"
+        out["kernel"] = "k_tile<float,8>" if st["blk_variant"] == -1 else "k_step_blk<float,8>"
         out["blk_variant"] = st["blk_variant"]
         out["timing"] = f"{reps} filter applications of {wl.L} steps, CUDA events on the library stream, after one warm"
     return out
@@ -634,10 +649,11 @@ def run_kes(args):
 
     # roofline of the fused step kernel, timed by the library's CUDA events on its stream
     step_ms = stats["filter_ms"] / max(stats["filter_steps"], 1)
-    bytes_step = K.kes_step_bytes(h, b, 1)
+    staged = stats["step_variant"] == -1
+    bytes_step = step_bytes(K, h, problems, wl.precision, b, 1, wl.L, staged)
     achieved = bytes_step / (step_ms / 1e3) / 1e9
     peak, peak_src = load_peak()
-    traffic = profiled_traffic(args.workload, STEP_KERNEL_SRC if b == 1 else BLOCK_KERNEL_SRC)
+    traffic = profiled_traffic(args.workload, STEP_KERNEL_SRC if b == 1 else BLOCK_KERNEL_SRC) if staged else None
 
     # several intervals from one trajectory: the same block filtered with F weight tables
     multi = None
@@ -652,7 +668,7 @@ def run_kes(args):
             K.kes_filter_apply(h, R0_dev, out, b)
         st = K.kes_get_stats(h)
         fms = st["filter_ms"] / reps
-        bF = K.kes_step_bytes(h, b, F)
+        bF = step_bytes(K, h, problems, wl.precision, b, F, wl.L, staged)
         multi = {"F": F, "b": b, "L": wl.L, "ms_per_filter": fms,
                  "value": n * b * wl.L / (fms / 1e3) / 1e9, "unit": METRIC,
                  "step_us": 1e3 * fms / wl.L, "achieved_gbs": bF / (fms / wl.L / 1e3) / 1e9,
@@ -768,7 +784,8 @@ def run_kes(args):
                    "l2": "inputs larger than L2 (matrix > 129 MB)"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
-                     "kernel": ("k_step_f64" if wl.precision == "fp64" else "k_step_f32") if b == 1
+                     "kernel": f"k_tile<{'double' if wl.precision == 'fp64' else 'float'},{b}>" if staged
+                     else ("k_step_f64" if wl.precision == "fp64" else "k_step_f32") if b == 1
                      else ("k_step_blk<double>" if wl.precision == "fp64" else "k_step_blk<float>"),
                      "step_variant": stats["step_variant"] if b == 1 else stats["blk_variant"],
                      "step_grid": stats["step_grid"] if b == 1 else stats["blk_grid"],
