@@ -158,7 +158,8 @@ typedef struct kes_stats {
   double filter_ms;         /* device time of the filter applications (CUDA events on the context stream) */
   double solve_other_ms;    /* device time of orthogonalisation, projection and residuals */
   int64_t bytes_per_step;   /* algorithmic HBM bytes of one fused step (see kes_step_bytes) */
-  int32_t step_variant;     /* launch shape of the step kernel in use, -1: the staged kernels */
+  int32_t step_variant;     /* launch shape of the step kernel in use, -1: the staged kernels (single filters of such a
+                               context may run as another kernel, see kes_filter_kernel) */
   int32_t step_grid;        /* its grid size in blocks */
   int32_t blk_variant;      /* launch shape of the block (SpMM) step kernel, -1 for single-vector contexts and the
                                staged kernels */
@@ -276,6 +277,15 @@ kes_status kes_sym_eig(int32_t k, const double* A, double* w, double* V);
 /* kes_launch_shapes: the number of launch shapes of the single-vector step kernel
    (kes_opts.step_variant) and of the block step kernel (kes_opts.blk_variant). */
 void kes_launch_shapes(int32_t* n_step, int32_t* n_block);
+/* kes_filter_kernel: what ran the context's last filter application, also inside a solve (the results
+   do not depend on it): one of enum kes_kernel. */
+enum kes_kernel {
+  KES_KERNEL_NONE = 0,     /* no filter application yet */
+  KES_KERNEL_SHAPES = 1,   /* one launch per step, a launch shape of the register-staged step kernels */
+  KES_KERNEL_STAGED = 2,   /* one launch per step, the staged step kernels */
+  KES_KERNEL_RESIDENT = 3  /* one launch for all steps (small matrices) */
+};
+int32_t kes_filter_kernel(const kes_ctx* ctx);
 /* kes_step_bytes: algorithmic HBM bytes of one fused leapfrog step of this context for b vectors
    and F intervals (every matrix entry, row pointer and per-row vector read or written once; an
    entry is its value plus a 2-byte column difference when the compact index is in use, else a

@@ -28,7 +28,8 @@ __all__ = [
     "Context", "header_functions", "kes_filter_apply_noalloc", "KES_NOALLOC_MAX_N",
     "kes_create_batch", "kes_mesh_count", "kes_estimate_omega_max_batch", "kes_set_filters_batch",
     "kes_block_krylov_solve", "kes_set_weights", "kes_alpha_gaussian", "kes_filter_apply_columns",
-    "kes_alpha_triangle", "kes_weights_response", "kes_launch_shapes", "kes_subspace_solve",
+    "kes_alpha_triangle", "kes_weights_response", "kes_launch_shapes", "kes_subspace_solve", "kes_filter_kernel",
+    "KES_KERNEL_NONE", "KES_KERNEL_SHAPES", "KES_KERNEL_STAGED", "KES_KERNEL_RESIDENT",
 ]
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -45,6 +46,7 @@ KES_PREC_FP64, KES_PREC_FP32 = 0, 1
 KES_MEM_DEVICE, KES_MEM_HOST = 0, 1
 KES_STEPPER_LEAPFROG, KES_STEPPER_LEAPFROG4 = 0, 1
 KES_REFINE_FP64, KES_REFINE_F32X2 = 0, 1
+KES_KERNEL_NONE, KES_KERNEL_SHAPES, KES_KERNEL_STAGED, KES_KERNEL_RESIDENT = 0, 1, 2, 3
 
 
 class KesError(RuntimeError):
@@ -124,6 +126,7 @@ _sig = {
     "kes_alpha_gaussian": (C.c_int, [C.c_double, C.c_double, C.c_double, C.c_int32, _P]),
     "kes_alpha_triangle": (C.c_int, [C.c_double, C.c_double, C.c_double, C.c_int32, _P]),
     "kes_weights_response": (C.c_int, [_P, C.c_double, C.c_int32, _P, C.c_int64, _P]),
+    "kes_filter_kernel": (C.c_int32, [_P]),
     "kes_launch_shapes": (None, [C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
 }
 for _name, (_res, _args) in _sig.items():
@@ -237,6 +240,11 @@ def kes_launch_shapes() -> tuple:
     a, b = C.c_int32(), C.c_int32()
     lib.kes_launch_shapes(C.byref(a), C.byref(b))
     return a.value, b.value
+
+
+def kes_filter_kernel(ctx: int) -> int:
+    """What ran the context's last filter application (KES_KERNEL_*)."""
+    return lib.kes_filter_kernel(ctx)
 
 
 def kes_weights_response(alpha, tau: float, omega) -> np.ndarray:

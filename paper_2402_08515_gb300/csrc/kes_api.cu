@@ -276,7 +276,10 @@ void run_filter(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
   }
   cudaEvent_t e0 = c->get_event(), e1 = c->get_event();
   KES_CUDA(cudaEventRecord(e0, c->stream));
-  if (resident_filter(c, NB, fp64, cpt, steps, x2)) {
+  const bool resident = resident_filter(c, NB, fp64, cpt, steps, x2);
+  const bool staged = c->tiled && !many_tables(c, NB, fp64, cpt, x2);
+  c->filter_kernel = resident ? KES_KERNEL_RESIDENT : staged ? KES_KERNEL_STAGED : KES_KERNEL_SHAPES;
+  if (resident) {
     launch_resident(c->A, c->resident, c->resident_range, fp64, fp64 && c->fold64, c->stream, NB, c->tau2m64,
                     c->stage_in, c->stage_out, c->F, c->alpha64, c->alpha_hi, c->alpha_lo, c->L, steps, cpt,
                     c->n_mesh(), c->d_flag);
@@ -1073,6 +1076,8 @@ void kes_launch_shapes(int32_t* n_step, int32_t* n_block) {
   if (n_step) *n_step = step_variant_count();
   if (n_block) *n_block = blk_variant_count();
 }
+
+int32_t kes_filter_kernel(const kes_ctx* c) { return c ? c->filter_kernel : KES_KERNEL_NONE; }
 
 int64_t kes_step_bytes(const kes_ctx* c, int32_t b, int32_t F) {
   if (!c || b < 1 || F < 1) return -1;
