@@ -2,7 +2,9 @@
 // lie in a few contiguous runs of rows, and the runs, the entries' places in them and the order
 // of the matrix values are laid out here, once per context.
 #include <algorithm>
+#include <atomic>
 #include <map>
+#include <new>
 
 #include "kes_internal.h"
 
@@ -108,6 +110,8 @@ bool build_tile_groups(const TileInput& in, TileLayout& out) {
   const int64_t ng = static_cast<int64_t>(out.groups.size());
   std::vector<std::vector<int32_t>> pats(ng);
   int64_t padded = 0, stored = 0;
+  // an exception must not leave a thread of a parallel region: it would end the process
+  std::atomic<bool> no_memory{false};
 #pragma omp parallel
   {
     std::vector<int32_t> tmp;
@@ -124,8 +128,14 @@ bool build_tile_groups(const TileInput& in, TileLayout& out) {
       }
       g.w = static_cast<int>(w);
       g.kind = 1;
-      if (w > 0)
-        group_pattern(in, g, in.mesh_row0[g.mesh], in.mesh_row0[g.mesh] + in.mesh_rows[g.mesh], pats[i], tmp);
+      if (w > 0) {
+        try {
+          group_pattern(in, g, in.mesh_row0[g.mesh], in.mesh_row0[g.mesh] + in.mesh_rows[g.mesh], pats[i], tmp);
+        } catch (const std::bad_alloc&) {
+          no_memory = true;
+          pats[i].clear();
+        }
+      }
       if (!pats[i].empty()) {
         g.kind = 0;
         g.w = static_cast<int>(pats[i].size());
@@ -133,6 +143,7 @@ bool build_tile_groups(const TileInput& in, TileLayout& out) {
       padded += static_cast<int64_t>(g.w) * g.rows;
     }
   }
+  if (no_memory) throw std::bad_alloc();
   // groups of uneven rows would be padded to their longest one: not worth staging
   if (padded > stored + stored / 8) return false;
   std::map<std::vector<int32_t>, int> known;
@@ -197,47 +208,55 @@ bool build_tiles(const TileInput& in, const TileLayout& lay, int R, TileHost& ou
   }
   if (head_at[nt] >= (int64_t(1) << 31)) return false;
   out.head.assign(head_at[nt], int4{0, 0, 0, 0});
-  bool fits = true;
+  std::atomic<bool> fits{true}, no_memory{false};
+  // the runs and places of an index tile; false: its columns are too scattered
+  auto index_tile = [&](int64_t t, std::vector<int32_t>& blocks) {
+    const Tile& tl = tiles[t];
+    blocks.clear();
+    int32_t last = -1;
+    for (int i = 0; i < tl.rows; ++i) {
+      const int64_t row = tl.row0 + i;
+      const int32_t* cs = in.col + in.slice_ptr[row / kSliceC] + row % kSliceC;
+      for (int32_t k = 0; k < in.len[row]; ++k) {
+        const int32_t b = cs[k * kSliceC] / kAlign;
+        if (b != last) blocks.push_back(b);
+        last = b;
+      }
+    }
+    for (int i = 0; i < tl.rows; i += kAlign) blocks.push_back(static_cast<int32_t>((tl.row0 + i) / kAlign));
+    std::sort(blocks.begin(), blocks.end());
+    blocks.erase(std::unique(blocks.begin(), blocks.end()), blocks.end());
+    std::vector<Run>& runs = runs_of[t];
+    for (int32_t b : blocks) add_range(runs, b * kAlign, (b + 1) * kAlign);
+    const int32_t xrows = place_runs(runs);
+    if (static_cast<int>(runs.size()) > kMaxRuns || xrows > kMaxStagedRows) return false;
+    const int w = tl.g->w;
+    for (int i = 0; i < tl.rows; ++i) {
+      const int64_t row = tl.row0 + i;
+      const int32_t* cs = in.col + in.slice_ptr[row / kSliceC] + row % kSliceC;
+      uint16_t* dst =
+          reinterpret_cast<uint16_t*>(&out.head[head_at[t] + 2]) + static_cast<int64_t>(i / kSliceC) * w * kSliceC;
+      const int32_t own = find_row(runs, static_cast<int32_t>(row));
+      for (int k = 0; k < w; ++k)
+        dst[quad_pos(w, k, i % kSliceC)] =
+            static_cast<uint16_t>(k < in.len[row] ? find_row(runs, cs[k * kSliceC]) : own);
+    }
+    return true;
+  };
 #pragma omp parallel
   {
     std::vector<int32_t> blocks;
-#pragma omp for schedule(dynamic, 64) reduction(&& : fits)
+#pragma omp for schedule(dynamic, 64)
     for (int64_t t = 0; t < nt; ++t) {
-      const Tile& tl = tiles[t];
-      if (tl.g->kind != 1) continue;
-      blocks.clear();
-      int32_t last = -1;
-      for (int i = 0; i < tl.rows; ++i) {
-        const int64_t row = tl.row0 + i;
-        const int32_t* cs = in.col + in.slice_ptr[row / kSliceC] + row % kSliceC;
-        for (int32_t k = 0; k < in.len[row]; ++k) {
-          const int32_t b = cs[k * kSliceC] / kAlign;
-          if (b != last) blocks.push_back(b);
-          last = b;
-        }
-      }
-      for (int i = 0; i < tl.rows; i += kAlign) blocks.push_back(static_cast<int32_t>((tl.row0 + i) / kAlign));
-      std::sort(blocks.begin(), blocks.end());
-      blocks.erase(std::unique(blocks.begin(), blocks.end()), blocks.end());
-      std::vector<Run>& runs = runs_of[t];
-      for (int32_t b : blocks) add_range(runs, b * kAlign, (b + 1) * kAlign);
-      const int32_t xrows = place_runs(runs);
-      if (static_cast<int>(runs.size()) > kMaxRuns || xrows > kMaxStagedRows) {
-        fits = false;
-        continue;
-      }
-      const int w = tl.g->w;
-      for (int i = 0; i < tl.rows; ++i) {
-        const int64_t row = tl.row0 + i;
-        const int32_t* cs = in.col + in.slice_ptr[row / kSliceC] + row % kSliceC;
-        uint16_t* dst = reinterpret_cast<uint16_t*>(&out.head[head_at[t] + 2]) + static_cast<int64_t>(i / kSliceC) * w * kSliceC;
-        const int32_t own = find_row(runs, static_cast<int32_t>(row));
-        for (int k = 0; k < w; ++k)
-          dst[quad_pos(w, k, i % kSliceC)] =
-              static_cast<uint16_t>(k < in.len[row] ? find_row(runs, cs[k * kSliceC]) : own);
+      if (tiles[t].g->kind != 1 || !fits || no_memory) continue;  // one tile that does not fit settles it
+      try {
+        if (!index_tile(t, blocks)) fits = false;
+      } catch (const std::bad_alloc&) {
+        no_memory = true;
       }
     }
   }
+  if (no_memory) throw std::bad_alloc();
   if (!fits) return false;
   std::vector<const PatRuns*> pat_of(nt, nullptr);
   for (int64_t t = 0; t < nt; ++t) {
