@@ -114,6 +114,7 @@ _sig = {
     "kes_get_stats": (C.c_int, [_P, C.POINTER(KesStats)]),
     "kes_reset_stats": (C.c_int, [_P]),
     "kes_filter_apply_noalloc": (C.c_int, [C.c_int64, _P, _P, _P, _P, _P, C.c_int32, _P, _P, _P]),
+    "kes_filter_apply_noalloc_sized": (C.c_int, [C.c_int64, C.c_int64, _P, _P, _P, _P, _P, C.c_int32, _P, _P, _P]),
     "kes_create_batch": (C.c_int, [C.POINTER(_P), C.c_int32, _P, _P, _P, _P, _P, C.POINTER(KesOpts)]),
     "kes_mesh_count": (C.c_int32, [_P]),
     "kes_estimate_omega_max_batch": (C.c_int, [_P, C.c_int32, _P, _P, _P]),
@@ -468,8 +469,9 @@ def kes_filter_apply_noalloc(n, row_ptr, col, val, tau2m, alpha, L, r_in, r_out,
         if len(devs) != 1 or col.numel() != val.numel():
             raise KesError(-1, "kes_filter_apply_noalloc: tensors on several devices, or col and val differ in length")
         torch.cuda.set_device(devs.pop())
-    _check(lib.kes_filter_apply_noalloc(n, _ptr(row_ptr), _ptr(col), _ptr(val), _ptr(tau2m), _ptr(alpha),
-                                        L, _ptr(r_in), _ptr(r_out), stream), "kes_filter_apply_noalloc")
+    nnz = col.numel() if isinstance(col, torch.Tensor) else -1
+    _check(lib.kes_filter_apply_noalloc_sized(n, nnz, _ptr(row_ptr), _ptr(col), _ptr(val), _ptr(tau2m), _ptr(alpha),
+                                              L, _ptr(r_in), _ptr(r_out), stream), "kes_filter_apply_noalloc")
 
 
 # ------------------------------------------------------------------ convenience

@@ -127,3 +127,65 @@ def test_noalloc_rejects_sizes_beyond_its_scratch_and_bad_tensors():
             K.kes_filter_apply_noalloc(n, args["row_ptr"], args["col"], args["val"], args["tau2m"], args["alpha"],
                                        L, args["r_in"], args["r_out"], None)
         assert e.value.status == -1
+
+
+def _rows_of(n, kind, seed):
+    """A seeded weighted graph Laplacian plus a small diagonal, with rows of a kind, and random lumped masses."""
+    rng = np.random.default_rng(seed)
+    on = np.ones(n, dtype=bool)
+    if kind == "uneven":      # short rows, some of thousands of entries, and whole groups of rows without any
+        on = ((np.arange(n) // 150) % 5 != 3) & (np.arange(n) < max(1, n - 200))
+        hubs, reach = rng.choice(n, max(1, n // 500), replace=False), 3
+        deg = rng.integers(min(n, 1500) // 2, min(n, 5000), len(hubs))
+    elif kind == "long":      # one long row in groups of few entries
+        hubs, reach = np.arange(11, n, 97), 1
+        deg = np.full(len(hubs), 300)
+    else:                     # about so many entries in every row
+        hubs, deg, reach = np.zeros(0, int), np.zeros(0, int), int(kind) // 2
+    I = np.r_[np.repeat(np.arange(n), reach), np.repeat(hubs, deg)]
+    J = np.r_[(np.arange(n)[:, None] + np.arange(1, reach + 1)).ravel(), rng.integers(0, n, int(deg.sum()))]
+    keep = (J < n) & (I != J) & (rng.random(len(I)) < 0.9)
+    keep[keep] &= on[I[keep]] & on[J[keep]]
+    I, J = I[keep], J[keep]
+    w = 0.5 + rng.random(len(I))
+    W = sp.coo_matrix((np.r_[w, w], (np.r_[I, J], np.r_[J, I])), shape=(n, n)).tocsr()
+    S = (sp.diags(np.asarray(W.sum(axis=1)).ravel() + 0.01 * on) - W).tocsr()
+    S.eliminate_zeros()
+    S.sort_indices()
+    return S, rng.uniform(0.5, 2.0, n)
+
+
+# groups of 128 rows are divided over 8 blocks up to 9,728 rows, 4 up to 19,456, 2 up to 38,912; a matrix of 20,000 rows
+# or more of 48 entries on average runs with its own kernel where the caller gives the number of entries
+@pytest.mark.parametrize("n,kind", [(1, "1"), (129, "long"), (5003, "uneven"), (30011, "uneven"), (4001, "long"),
+                                    (700, "81"), (4999, "25"), (12001, "31"), (12001, "47"), (25001, "31"),
+                                    (25001, "47"), (50003, "41"), (50003, "31"), (50003, "81"), (20001, "61"),
+                                    (2000, "600")])
+@pytest.mark.parametrize("L", [1, 2, 20])
+def test_noalloc_takes_rows_of_every_width(n, kind, L):
+    import torch
+    S, m = _rows_of(n, kind, 7)
+    gersh = float(np.max(np.asarray(abs(S).sum(axis=1)).ravel() / m))  # >= omega_max^2
+    tau = 0.9 * 2 / np.sqrt(gersh)
+    alpha = O.alpha_table(0.2 / tau, 0.5 / tau, tau, L)
+    r = start_vectors(n, 1, 32)
+    ref = O.filter_apply(S, m, r[0], tau, alpha)
+    dev = torch.device("cuda", 0)
+    arrays = [torch.from_numpy(np.ascontiguousarray(a)).to(dev) for a in
+              (S.indptr.astype(np.int64), S.indices.astype(np.int32), S.data, tau * tau / m, alpha)]
+    r_in = torch.from_numpy(r[0]).to(dev)
+    stream = torch.cuda.current_stream(dev).cuda_stream
+    # the tolerance counts the roundings of rows of up to 16 entries: one more per entry, each of a partial sum of the
+    # same size, so the random walk of a wider row is longer by the root of its width over 16
+    wide = np.sqrt(max(1.0, np.diff(S.indptr).max() / 16))
+    for sized in (True, False):  # the binding gives the number of entries; the C entry without it
+        r_out = torch.full((n,), float("nan"), dtype=torch.float64, device=dev)
+        if sized:
+            K.kes_filter_apply_noalloc(n, *arrays, L, r_in, r_out, stream)
+        else:
+            assert K.lib.kes_filter_apply_noalloc(n, *[a.data_ptr() for a in arrays], L, r_in.data_ptr(),
+                                                  r_out.data_ptr(), stream) == 0
+        torch.cuda.synchronize(dev)
+        got = r_out.cpu().numpy()
+        assert np.isfinite(got).all()
+        assert filter_error(got, ref, r, m, alpha) <= wide * filter_tol(L, "fp64"), sized
