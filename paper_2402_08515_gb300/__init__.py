@@ -29,7 +29,7 @@ __all__ = [
     "kes_create_batch", "kes_mesh_count", "kes_estimate_omega_max_batch", "kes_set_filters_batch",
     "kes_block_krylov_solve", "kes_set_weights", "kes_alpha_gaussian", "kes_filter_apply_columns",
     "kes_alpha_triangle", "kes_weights_response", "kes_launch_shapes", "kes_subspace_solve", "kes_filter_kernel",
-    "KES_KERNEL_NONE", "KES_KERNEL_SHAPES", "KES_KERNEL_STAGED", "KES_KERNEL_RESIDENT",
+    "kes_set_wait_limit", "KES_KERNEL_NONE", "KES_KERNEL_SHAPES", "KES_KERNEL_STAGED", "KES_KERNEL_RESIDENT",
 ]
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -128,6 +128,7 @@ _sig = {
     "kes_alpha_triangle": (C.c_int, [C.c_double, C.c_double, C.c_double, C.c_int32, _P]),
     "kes_weights_response": (C.c_int, [_P, C.c_double, C.c_int32, _P, C.c_int64, _P]),
     "kes_filter_kernel": (C.c_int32, [_P]),
+    "kes_set_wait_limit": (C.c_int, [_P, C.c_int32]),
     "kes_launch_shapes": (None, [C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
 }
 for _name, (_res, _args) in _sig.items():
@@ -246,6 +247,11 @@ def kes_launch_shapes() -> tuple:
 def kes_filter_kernel(ctx: int) -> int:
     """What ran the context's last filter application (KES_KERNEL_*)."""
     return lib.kes_filter_kernel(ctx)
+
+
+def kes_set_wait_limit(ctx: int, polls: int) -> None:
+    """Polls that a device-side wait takes before it gives up (KES_ERR_TIMEOUT); -1: the default, about 1.5 s."""
+    _check(lib.kes_set_wait_limit(ctx, int(polls)), "kes_set_wait_limit")
 
 
 def kes_weights_response(alpha, tau: float, omega) -> np.ndarray:

@@ -38,7 +38,8 @@ namespace {
 constexpr int kGroupWarps = 8;      // warps that share a tile
 constexpr int kMaxStages = 6;
 constexpr int kTileSmem = 220 * 1024;  // bytes of shared memory a block may take
-constexpr int kWaitLimit = 1 << 20; // polls of a wait (each suspends the warp for a while) before it gives up
+// Polls of a wait before it gives up: 1.5 us each on GB300 (the hardware suspends the warp), 1.5 seconds in all.
+constexpr int kWaitLimit = 1 << 20;
 
 struct TileArgs {
   TileSet ts;
@@ -59,6 +60,7 @@ struct TileArgs {
   int keep, chained;
   int stages, stage_bytes, off_prev, off_own, off_acc, off_val, off_head;
   int* flag;
+  int waits;          // polls of a wait before it gives up
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -74,8 +76,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // Waits for the phase of that parity to complete; false once the limit is reached.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < kWaitLimit; ++i) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int limit) {
+  for (int i = 0; i < limit; ++i) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
@@ -218,7 +220,7 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
       }
     };
     auto wait_empty = [&]() {
-      return n < stages || mbar_wait(smem_addr(&bars[kMaxStages + st]), phase ^ 1);
+      return n < stages || mbar_wait(smem_addr(&bars[kMaxStages + st]), phase ^ 1, a.waits);
     };
     const int M = a.ts.max_runs + 2;
     if (((warp - kGroupWarps * GROUPS) & 1) == 0) {
@@ -288,9 +290,9 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
       }
     }
     if (!ok && lane == 0) atomicOr(a.flag, 2);
-    // the copies still in flight write this block's shared memory
+    // the copies still in flight write this block's shared memory: they land whatever limit was set
     for (int i = n - GROUPS; i >= 0 && i >= n - stages; i -= GROUPS)
-      mbar_wait(smem_addr(&bars[i % stages]), (i / stages) & 1);
+      mbar_wait(smem_addr(&bars[i % stages]), (i / stages) & 1, kWaitLimit);
     return;
   }
 
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
   int st = grp;  // stages >= GROUPS
   uint32_t phase = 0;
   for (int n = grp; n < mine; n += GROUPS) {
-    if (!mbar_wait(smem_addr(&bars[st]), phase)) {
+    if (!mbar_wait(smem_addr(&bars[st]), phase, a.waits)) {
       if (lane == 0) atomicOr(a.flag, 2);
       break;
     }
@@ -664,6 +666,7 @@ void launch_tile_step(const TileStep& p, cudaStream_t st) {
   a.last = p.last;
   a.fold2 = p.fold2;
   a.flag = p.flag;
+  a.waits = p.waits >= 0 ? p.waits : kWaitLimit;
   a.stages = f.stages;
   a.chained = p.chained;
   a.keep = keep_in_l2(p, size);

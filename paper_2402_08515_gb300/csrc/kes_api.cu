@@ -114,6 +114,7 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
     p.L = L;
     p.cpt = cpt;
     p.flag = c->d_flag;
+    p.waits = c->waits;
     int next = p.type == kTileF64 ? 0 : 1;  // first weighted term not yet in the accumulators
     for (int s = 0; s < steps; ++s) {
       p.x = s == 0 ? start : U[(s - 1) & 1];
@@ -1075,6 +1076,16 @@ kes_status kes_sync(kes_ctx* ctx) {
 void kes_launch_shapes(int32_t* n_step, int32_t* n_block) {
   if (n_step) *n_step = step_variant_count();
   if (n_block) *n_block = blk_variant_count();
+}
+
+kes_status kes_set_wait_limit(kes_ctx* c, int32_t polls) {
+  if (!c || polls < -1) return KES_ERR_ARG;
+  return guarded([&]() -> kes_status {
+    c->sync();
+    c->waits = polls;
+    c->drop_graphs();  // the limit is a parameter of their kernels
+    return KES_OK;
+  });
 }
 
 int32_t kes_filter_kernel(const kes_ctx* c) { return c ? c->filter_kernel : KES_KERNEL_NONE; }

@@ -121,3 +121,26 @@ def test_eight_columns_with_several_tables(b, use_graph):
 def test_the_lines_between_the_kernels(precision, b, F, n, reach, kernel):
     p = _lattice(n, reach)
     assert _both(p, b, F, 6, precision=precision, tau=0.3) == getattr(K, f"KES_KERNEL_{kernel}")
+
+
+@pytest.mark.parametrize("precision,b,opts", [("fp64", 1, {}), ("fp32", 8, {}), ("fp32", 2, dict(use_graph=False)),
+                                              ("fp64", 4, dict(stepper="leapfrog4"))])
+def test_a_wait_that_runs_out_is_an_error_and_the_context_stays_usable(precision, b, opts):
+    """With a limit of no polls every wait of the staged steps gives up: the copies under way still land, the call says
+    KES_ERR_TIMEOUT, and with the default limit the same context filters as if nothing had been."""
+    p = box_grid((43, 31, 29))
+    R = start_vectors(p.n, b, 11)
+    with K.Context(p, precision=precision, block_b=b, **opts) as c:
+        ref, kernel = _apply(c, p.n, b, 1, 8, 0.004)
+        assert kernel == K.KES_KERNEL_STAGED
+        K.kes_set_wait_limit(c.handle, 0)
+        with pytest.raises(K.KesError) as e:
+            K.kes_filter_apply(c.handle, R, np.zeros((1, b, p.n)), b)
+        assert e.value.status == -6
+        with pytest.raises(K.KesError) as e:
+            K.kes_set_wait_limit(c.handle, -2)
+        assert e.value.status == -1
+        K.kes_set_wait_limit(c.handle, -1)
+        out = np.zeros((1, b, p.n))
+        K.kes_filter_apply(c.handle, R, out, b)
+        np.testing.assert_array_equal(out, ref)
