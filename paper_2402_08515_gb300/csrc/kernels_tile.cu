@@ -597,17 +597,28 @@ void launch_groups(TileArgs a, int grid, cudaStream_t st) {
 // Three groups of warps where two stages for each fit, else two (128^3 cells, one column: FP32,
 // six stages, 22.7 us a step with three and 23.8 us with two; FP64, four stages of 45 KB, 59.2 us
 // with two groups; three (78 us when two took 62.7) leave none to be filled while the others are in use).
+// Four FP32 columns take two groups all the same: with three, 64 registers a thread hold a row's sums
+// and loads only with spills (300 thousand rows, us a step with three / two groups: 7 entries a row in 2D
+// 9.5 / 7.6, 25 entries 15.9 / 13.1; 970 thousand rows of a tube 34.4 / 29.5).
+constexpr int groups_of(int stages, int value_bytes, int NB) {
+  return stages >= 6 && !(value_bytes == 4 && NB == 4) ? 3 : 2;
+}
 template <typename T, int NB, int MODE>
 void launch_one(const TileArgs& a, int grid, cudaStream_t st) {
   if constexpr (std::is_same<T, double>::value && MODE == 0) {
     if (a.fold2) {
-      if (a.stages >= 6) launch_groups<T, NB, MODE, 3, true>(a, grid, st);
+      if (groups_of(a.stages, sizeof(T), NB) == 3) launch_groups<T, NB, MODE, 3, true>(a, grid, st);
       else launch_groups<T, NB, MODE, 2, true>(a, grid, st);
       return;
     }
   }
-  if (a.stages >= 6) launch_groups<T, NB, MODE, 3, false>(a, grid, st);
-  else launch_groups<T, NB, MODE, 2, false>(a, grid, st);
+  if constexpr (groups_of(6, sizeof(T), NB) == 3) {
+    if (a.stages >= 6) {
+      launch_groups<T, NB, MODE, 3, false>(a, grid, st);
+      return;
+    }
+  }
+  launch_groups<T, NB, MODE, 2, false>(a, grid, st);
 }
 
 template <typename T, int MODE>
@@ -636,6 +647,12 @@ bool keep_in_l2(const TileStep& p, int size) {
 
 int tile_stages(int R, int max_xrows, int max_w, int max_head, int row_bytes, int value_bytes, int NB, bool ho) {
   return fit_stage(R, max_xrows, max_w, max_head, row_bytes, value_bytes, NB, ho, kTileSmem).stages;
+}
+
+int tile_busy_warps(int R, int stages, int value_bytes, int NB) {
+  const int columns = std::min(NB, 16 / value_bytes);  // of a lane (CPL)
+  const int passes = R * (NB / columns) / kSliceC;     // of a warp over the tile's rows
+  return std::min(kGroupWarps, passes) * groups_of(stages, value_bytes, NB);
 }
 
 void launch_tile_step(const TileStep& p, cudaStream_t st) {

@@ -68,13 +68,33 @@ namespace {
 // Largest stable tau * omega of the context's stepper.
 double cfl_bound(const kes_ctx* c) { return c->opts.stepper == KES_STEPPER_LEAPFROG4 ? 2.0 * std::sqrt(3.0) : 2.0; }
 
+// Whether the rows are too narrow for the staged steps to gain in FP32: a row's share of the copies and barriers
+// costs more than the few gathers that they save while the matrix stays in L2 (us a step, launch shapes / staged, 300
+// thousand rows: 3 entries a row, 1 column 3.5 / 4.1, 8 columns 7.2 / 8.7; 7 entries, 8 columns 8.9 / 10.4; with 15
+// entries 1 column 6.8 / 5.1, 8 columns 12.9 / 13.1). The line lies higher for columns with a table each (47 thousand
+// rows of 7 entries 3.6 / 3.4, 65 thousand 3.7 / 4.1) and lower for 1 column (7 entries in 3D: 97 thousand rows 2.7 / 2.8,
+// 300 thousand 4.8 / 4.5, 1 million 16.3 / 12.9). Matrices of up to 20 thousand rows mostly run as the resident filter.
+bool too_narrow(const kes_ctx* c, int NB, int cpt) {
+  if (!c->narrow) return false;
+  const int64_t from = cpt > 0 ? 56 * 1024 : 20 * 1024, to = int64_t(1) << (NB == 1 && c->nnz_q > 4 * c->n_pad ? 18 : 19);
+  return c->n_pad >= from && c->n_pad < to;
+}
+bool staged_width(const kes_ctx* c, int type, int NB, int cpt) {
+  return c->has_tiles(type, NB) && !(type == kTileF32 && too_narrow(c, NB, cpt));
+}
+
 // Whether a staged context runs this filter with the register-staged block kernel all the same:
 // eight FP32 columns that each add to several weight tables. The staged step keeps one table's
 // accumulators in its stages; the others' 1 KB a row of 16 is latency that its 16 computing warps
 // do not hide (96^3 cells, us a step: 2 tables 41.6 against 43.9 staged, 4 tables 53.9 against
 // 64.5; with one 35.1 against 33.1, and narrower blocks and FP64 are faster staged with 4, too).
 bool many_tables(const kes_ctx* c, int NB, bool fp64, int cpt, bool x2) {
-  return c->tiled && !fp64 && !x2 && NB == 8 && cpt == 0 && c->F > 1 && c->opts.stepper == KES_STEPPER_LEAPFROG;
+  return staged_width(c, kTileF32, 8, 0) && !fp64 && !x2 && NB == 8 && cpt == 0 && c->F > 1 &&
+         c->opts.stepper == KES_STEPPER_LEAPFROG;
+}
+// The kernel of a filter that does not run as the resident one.
+bool staged_filter(const kes_ctx* c, int NB, bool fp64, int cpt, bool x2) {
+  return staged_width(c, x2 ? kTileX2 : fp64 ? kTileF64 : kTileF32, NB, cpt) && !many_tables(c, NB, fp64, cpt, x2);
 }
 constexpr int kManyTablesShape = 13;  // the shape that the autotuner picks for it on the meshes at hand
 
@@ -88,7 +108,7 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
   const bool ho = c->opts.stepper == KES_STEPPER_LEAPFROG4;
   const int L = c->L, F = c->F;  // L: the tables' length (their stride is L + 1)
   const int64_t stride = c->n_pad * NB;
-  if (c->tiled && !many_tables(c, NB, fp64, cpt, x2)) {
+  if (staged_filter(c, NB, fp64, cpt, x2)) {
     TileStep p;
     p.type = x2 ? kTileX2 : fp64 ? kTileF64 : kTileF32;
     p.ts = c->tiles[c->tile_of[p.type][log2_nb(NB)]];
@@ -185,7 +205,7 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
   } else {
     const SellDev A32 = c->step_A32();
     LaunchCfg cfg = c->cfg;
-    if (c->tiled) {
+    if (many_tables(c, NB, fp64, cpt, x2)) {
       cfg.variant_blk = kManyTablesShape;
       cfg.grid_blk = cfg.n_sm * blk_blocks_per_sm(true, NB, kManyTablesShape, cfg.block_step);
     }
@@ -227,32 +247,36 @@ bool resident_filter(const kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
   return resident_fits(c->resident, fp64, cpt ? 1 : c->F, c->n_mesh(), steps);
 }
 
-// The FP64 step kernels in a context of the FP32 form (used by the FP64 refinement).
-void ensure_fp64_state(kes_ctx* c) {
-  if (!c->U64[0])
-    for (int j = 0; j < 2; ++j) c->U64[j] = c->dzero_n<double>(c->n_pad * c->NBcap);
-  if (c->tiled) {
-    if (!c->q64) {
-      c->q64 = c->dzero_n<double>(c->nnz_q);
-      launch_scale_tiles(c->A, c->slice_rec, c->tile_pat, c->cfg.n_sm, c->stream, c->tau2m64, c->q64, nullptr,
-                         c->fold64);
-      KES_CHECK_LAUNCH();
-    }
-  } else if (!c->step64) {
+// The FP64 step values in the order that the kernels of a width read.
+void ensure_fp64_values(kes_ctx* c, bool tiles) {
+  if (tiles && !c->q64) {
+    c->q64 = c->dzero_n<double>(c->nnz_q);
+    launch_scale_tiles(c->A, c->slice_rec, c->tile_pat, c->cfg.n_sm, c->stream, c->tau2m64, c->q64, nullptr,
+                       c->fold64);
+    KES_CHECK_LAUNCH();
+  } else if (!tiles && !c->step64) {
     c->step64 = c->dzero_n<double>(c->nnz_pad);
     launch_scale_values(c->A, c->cfg, c->stream, c->tau2m64, c->step64, nullptr, nullptr, nullptr, c->fold64);
     KES_CHECK_LAUNCH();
   }
 }
 
+// The FP64 step kernels in a context of the FP32 form (used by the FP64 refinement).
+void ensure_fp64_state(kes_ctx* c, int NB) {
+  if (!c->U64[0])
+    for (int j = 0; j < 2; ++j) c->U64[j] = c->dzero_n<double>(c->n_pad * c->NBcap);
+  ensure_fp64_values(c, c->has_tiles(kTileF64, NB));
+}
+
 // The FP32-pair steps in a context of the FP32 form: step values split from the FP64 ones
 // (again after a filter change rescaled those) and the pair state.
-void ensure_x2_state(kes_ctx* c) {
-  ensure_fp64_state(c);
-  const int64_t count = c->tiled ? c->nnz_q : c->nnz_pad;
+void ensure_x2_state(kes_ctx* c, int NB) {
+  const bool tiles = c->has_tiles(kTileX2, NB);  // the same for every width
+  ensure_fp64_values(c, tiles);
+  const int64_t count = tiles ? c->nnz_q : c->nnz_pad;
   if (!c->step2) c->step2 = c->dzero_n<float2>(count);
   if (!c->step2_fresh) {
-    launch_split_values(c->stream, count, c->tiled ? c->q64 : c->step64, c->step2);
+    launch_split_values(c->stream, count, tiles ? c->q64 : c->step64, c->step2);
     KES_CHECK_LAUNCH();
     c->step2_fresh = true;
   }
@@ -269,8 +293,8 @@ void run_filter(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
   if (x2 && (NB < 2 || c->opts.precision != KES_PREC_FP32 || c->opts.stepper != KES_STEPPER_LEAPFROG))
     throw KesError{KES_ERR_UNSUPPORTED};
   if (steps <= 0 || steps > c->L) steps = c->L;
-  if (x2) ensure_x2_state(c);
-  else if (fp64) ensure_fp64_state(c);
+  if (x2) ensure_x2_state(c, NB);
+  else if (fp64) ensure_fp64_state(c, NB);
   if (c->opts.stepper == KES_STEPPER_LEAPFROG4) {  // stage buffers before any graph captures them
     if (fp64 && !c->V64) c->V64 = c->dzero_n<double>(c->n_pad * c->NBcap);
     if (!fp64 && !c->V32) c->V32 = c->dzero_n<float>(c->n_pad * c->NBcap);
@@ -278,7 +302,7 @@ void run_filter(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
   cudaEvent_t e0 = c->get_event(), e1 = c->get_event();
   KES_CUDA(cudaEventRecord(e0, c->stream));
   const bool resident = resident_filter(c, NB, fp64, cpt, steps, x2);
-  const bool staged = c->tiled && !many_tables(c, NB, fp64, cpt, x2);
+  const bool staged = staged_filter(c, NB, fp64, cpt, x2);
   c->filter_kernel = resident ? KES_KERNEL_RESIDENT : staged ? KES_KERNEL_STAGED : KES_KERNEL_SHAPES;
   if (resident) {
     launch_resident(c->A, c->resident, c->resident_range, fp64, fp64 && c->fold64, c->stream, NB, c->tau2m64,
@@ -502,18 +526,13 @@ void validate_csr(int64_t n, const int64_t* row_ptr, const int32_t* col, const d
 
 // The step kernels in use, for the statistics: a launch shape, or -1 for the staged ones.
 void shape_stats(kes_ctx* c) {
-  if (c->tiled) {
-    const int type = c->opts.precision == KES_PREC_FP32 ? kTileF32 : kTileF64;
-    c->stats.step_variant = c->stats.blk_variant = -1;
-    c->stats.step_grid = std::min(c->cfg.n_sm, c->tiles[c->tile_of[type][0]].n_tiles);
-    c->stats.blk_grid =
-        c->NBcap > 1 ? std::min(c->cfg.n_sm, c->tiles[c->tile_of[type][log2_nb(c->NBcap)]].n_tiles) : 0;
-    return;
-  }
-  c->stats.step_variant = c->cfg.variant;
-  c->stats.step_grid = c->cfg.grid_step;
-  c->stats.blk_variant = c->NBcap > 1 ? c->cfg.variant_blk : -1;
-  c->stats.blk_grid = c->NBcap > 1 ? c->cfg.grid_blk : 0;
+  const int type = c->own_type();
+  auto grid = [&](int NB) { return std::min(c->cfg.n_sm, c->tiles[c->tile_of[type][log2_nb(NB)]].n_tiles); };
+  const bool one = staged_width(c, type, 1, 0), blk = c->NBcap > 1 && staged_width(c, type, c->NBcap, 0);
+  c->stats.step_variant = one ? -1 : c->cfg.variant;
+  c->stats.step_grid = one ? grid(1) : c->cfg.grid_step;
+  c->stats.blk_variant = c->NBcap > 1 && !blk ? c->cfg.variant_blk : -1;
+  c->stats.blk_grid = blk ? grid(c->NBcap) : c->NBcap > 1 ? c->cfg.grid_blk : 0;
 }
 
 template <typename T>
@@ -524,8 +543,11 @@ T* upload(kes_ctx* c, const std::vector<T>& v) {
   return d;
 }
 
-// Lays the matrix out for the staged steps where it allows them: every tile's columns in a few
-// runs of rows, and at least two stages of every precision and block width in shared memory.
+// Lays the matrix out for the staged steps where it allows them: every tile's columns in a few runs of rows, and at
+// least four stages in shared memory of tiles large enough to keep four warps busy (FP32 pairs: at least two
+// stages). With fewer the launch shapes are faster: 125 entries a row, 300 thousand rows, us a step, shapes /
+// staged: FP64 1 column (tiles of 32 rows: two busy warps) 72.6 / 189.7, 4 columns (two stages) 273 / 350, FP32 4
+// columns (32 rows) 47.4 / 70.6; FP32 1 column (64 rows, four stages: four busy warps) 43.0 / 28.1.
 void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, const std::vector<int32_t>& cols,
                 const std::vector<int32_t>& lens) {
   std::vector<int64_t> row0, rows;
@@ -551,40 +573,48 @@ void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, co
     for (int64_t r : rows) n += (r + (kTileGroup >> i) - 1) / (kTileGroup >> i);
     return n;
   };
+  // in order of what the busiest block does, in rows: a tile's own cost counts as 96, and the
+  // first tile has to be there before anything starts
+  int order[4] = {0, 1, 2, 3};
+  auto cost = [&](int i) {
+    return (tiles_of(i) + c->cfg.n_sm - 1) / c->cfg.n_sm * ((kTileGroup >> i) + 96) + (kTileGroup >> i);
+  };
+  std::stable_sort(order, order + 4, [&](int a, int b) { return cost(a) < cost(b); });
   for (int type = 0; type < 3; ++type) {
     if (type != kTileF64 && !fp32) continue;
+    const int size = type == kTileF32 ? 4 : 8;
     for (int NB = type == kTileX2 ? 2 : 1; NB <= c->NBcap; NB *= 2) {
-      // in order of what the busiest block does, in rows: a tile's own cost counts as 96, and the
-      // first tile has to be there before anything starts
-      int order[4] = {0, 1, 2, 3};
-      auto cost = [&](int i) {
-        return (tiles_of(i) + c->cfg.n_sm - 1) / c->cfg.n_sm * ((kTileGroup >> i) + 96) + (kTileGroup >> i);
-      };
-      std::stable_sort(order, order + 4, [&](int a, int b) { return cost(a) < cost(b); });
-      int pick = -1;
-      for (int want = 4; want >= 2 && pick < 0; want -= 2)
-        for (int q = 0; q < 4 && pick < 0; ++q) {
-          const int i = order[q];
-          if (!tried[i]) {
-            tried[i] = true;
-            ok[i] = build_tiles(in, lay, kTileGroup >> i, built[i]);
-          }
-          if (!ok[i]) continue;
-          const int size = type == kTileF32 ? 4 : 8;
-          if (tile_stages(built[i].R, built[i].max_xrows, built[i].max_w, built[i].max_head, size * NB, size, NB, ho) >=
-              want)
-            pick = i;
+      auto stages_of = [&](int i) {
+        if (!tried[i]) {
+          tried[i] = true;
+          ok[i] = build_tiles(in, lay, kTileGroup >> i, built[i]);
         }
-      if (pick < 0) return;
+        return ok[i] ? tile_stages(built[i].R, built[i].max_xrows, built[i].max_w, built[i].max_head, size * NB, size, NB, ho)
+                     : 0;
+      };
+      int pick = -1, busy = 0;
+      for (int want = 4; want >= (type == kTileX2 ? 2 : 4) && pick < 0; want -= 2)
+        for (int q = 0; q < 4 && pick < 0; ++q)
+          if (stages_of(order[q]) >= want) pick = order[q];
+      // the pick may have few rows because the matrix has few; the largest tiles that fit tell
+      for (int i = 0; i < 4 && pick >= 0 && busy == 0; ++i)
+        if (const int stages = stages_of(i); stages >= 4) busy = tile_busy_warps(kTileGroup >> i, stages, size, NB);
+      if (type != kTileX2 && busy < 4) pick = -1;
       c->tile_of[type][log2_nb(NB)] = pick;
+      if (type == kTileX2 && pick < 0) {  // the pairs' values have one order for all widths
+        for (int& t : c->tile_of[type]) t = -1;
+        break;
+      }
     }
   }
   for (int type = 0; type < 3; ++type)
     for (int q = 0; q < 4; ++q) {
       const int i = c->tile_of[type][q];
+      if (i < 0) continue;
+      c->tiled = true;
       const TileHost& h = built[i];
       TileSet& ts = c->tiles[i];
-      if (!ok[i] || ts.seg) continue;
+      if (ts.seg) continue;
       ts.n_tiles = static_cast<int>(h.seg.size() / (h.max_runs + 2));
       ts.R = h.R;
       ts.max_xrows = h.max_xrows;
@@ -594,10 +624,14 @@ void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, co
       ts.seg = upload(c, h.seg);
       ts.head = upload(c, h.head);
     }
+  if (!c->tiled) return;
+  c->nnz_q = lay.n_values;
+  c->narrow = fp32 && !ho && lay.n_values <= 8 * c->n_pad;
+  c->shapes = false;
+  for (int NB = 1; NB <= c->NBcap; NB *= 2)
+    c->shapes = c->shapes || !staged_width(c, c->own_type(), NB, 0) || (NB > 1 && !staged_width(c, c->own_type(), NB, 1));
   c->slice_rec = upload(c, lay.slice_rec);
   c->tile_pat = upload(c, lay.pat);
-  c->nnz_q = lay.n_values;
-  c->tiled = true;
   c->sync();  // the host vectors go out of scope
 }
 
@@ -748,7 +782,7 @@ void build_context(kes_ctx* c, int nm, const int64_t* n, const int64_t* const* r
     int16_t* d_dcol = c->dalloc_n<int16_t>(nnz_pad);
     KES_CUDA(cudaMemcpyAsync(d_dcol, dcol.data(), nnz_pad * sizeof(int16_t), cudaMemcpyHostToDevice, c->stream));
     c->A.dcol = d_dcol;
-    if (!c->tiled) {
+    if (c->shapes) {
       // pair layout for the single-vector steps: entry k of lane l of slice s at
       // sp2[s] + 64 (k / 2) + 2 l + k % 2, odd widths padded with a zero entry per lane
       std::vector<int64_t> sp2(n_slices + 1, 0);
@@ -840,14 +874,17 @@ kes_status create_impl(kes_ctx** out, int32_t nm, const int64_t* n, const int64_
     c->fold64 = c->diag_in_rows && c->opts.stepper == KES_STEPPER_LEAPFROG;
     const int64_t np = c->n_pad, nb = c->NBcap;
     c->tau2m64 = c->dzero_n<double>(np);
+    bool own_staged = false;
+    for (int NB = 1; NB <= c->NBcap; NB *= 2)
+      own_staged = own_staged || staged_width(c, c->own_type(), NB, 0) || (NB > 1 && staged_width(c, c->own_type(), NB, 1));
     if (c->opts.precision == KES_PREC_FP32) {
-      if (c->tiled) c->q32 = c->dzero_n<float>(c->nnz_q);  // zero where a row lacks its pattern's entry
-      else c->step32 = c->dzero_n<float>(c->nnz_pad);
+      if (own_staged) c->q32 = c->dzero_n<float>(c->nnz_q);  // zero where a row lacks its pattern's entry
+      if (c->shapes) c->step32 = c->dzero_n<float>(c->nnz_pad);
       if (c->A.slice_ptr2) c->step32p = c->dzero_n<float>(c->nnz_pair);  // padding stays zero
       for (int j = 0; j < 3; ++j) c->U32[j] = c->dzero_n<float>(np * nb);
     } else {
-      if (c->tiled) c->q64 = c->dzero_n<double>(c->nnz_q);
-      else c->step64 = c->dzero_n<double>(c->nnz_pad);
+      if (own_staged) c->q64 = c->dzero_n<double>(c->nnz_q);
+      if (c->shapes) c->step64 = c->dzero_n<double>(c->nnz_pad);
       if (c->A.slice_ptr2 && c->fold64) c->step64p = c->dzero_n<double>(c->nnz_pair);  // padding stays zero
       for (int j = 0; j < 2; ++j) c->U64[j] = c->dzero_n<double>(np * nb);
     }
@@ -864,7 +901,7 @@ kes_status create_impl(kes_ctx** out, int32_t nm, const int64_t* n, const int64_
     c->cfg.variant_blk = c->opts.blk_variant;
     c->cfg.grid_blk =
         n_sm * blk_blocks_per_sm(fp32, c->NBcap > 1 ? c->NBcap : 2, c->opts.blk_variant, c->cfg.block_step);
-    if (c->opts.autotune && !c->tiled) tune_steps(c);
+    if (c->opts.autotune && c->shapes) tune_steps(c);
     c->sync();
     c->stats.bytes_per_step = kes_step_bytes(c, 1, 1);
     shape_stats(c);
@@ -936,14 +973,14 @@ kes_status set_weights_impl(kes_ctx* c, int32_t F, const double* alpha, const do
     }
     KES_CUDA(cudaMemcpyAsync(c->tau2m64, t2m.data(), c->n_pad * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     // the register-staged block kernel's values, where a filter may take it (many_tables)
-    if (c->tiled && !c->step32 && c->opts.precision == KES_PREC_FP32 && c->NBcap == 8 && F > 1 &&
+    if (!c->step32 && c->opts.precision == KES_PREC_FP32 && c->NBcap == 8 && F > 1 &&
         c->opts.stepper == KES_STEPPER_LEAPFROG)
       c->step32 = c->dzero_n<float>(c->nnz_pad);
     // step values A = -tau^2 M^{-1} S (the FP32 ones rounded once from the FP64 product)
     if (c->step64 || c->step32)
       launch_scale_values(c->A, c->cfg, c->stream, c->tau2m64, c->step64, c->step32, c->step64p, c->step32p,
                           c->fold64);
-    if (c->tiled)
+    if (c->q64 || c->q32)
       launch_scale_tiles(c->A, c->slice_rec, c->tile_pat, c->cfg.n_sm, c->stream, c->tau2m64, c->q64, c->q32,
                          c->fold64);
     c->step2_fresh = false;  // the FP32-pair values follow step64 at their next use

@@ -106,15 +106,19 @@ struct kes_ctx {
   int64_t nnz_pair = 0;           // entries of the pair layout (with its padding)
   // staged steps (kernels_tile.cu), where the matrix allows them and no launch shape was asked
   // for: the step values in the order of the tiles, one tile set per number of rows in use, and
-  // which of them a precision and block width takes
+  // which of them a precision and block width takes (-1: it runs as launch shapes, see plan_tiles)
   bool tiled = false;
+  bool narrow = false;            // FP32 leapfrog with few entries a row: not every width gains from the staged steps
+  bool shapes = true;             // filters of the context's own precision may run as launch shapes
   double* q64 = nullptr;
   float* q32 = nullptr;
   int64_t nnz_q = 0;
   int4* slice_rec = nullptr;
   int32_t* tile_pat = nullptr;
   kes::TileSet tiles[4];          // of 256, 128, 64 and 32 rows
-  int tile_of[3][4] = {};         // [TileType][log2 NB]
+  int tile_of[3][4] = {{-1, -1, -1, -1}, {-1, -1, -1, -1}, {-1, -1, -1, -1}};  // [TileType][log2 NB]
+  bool has_tiles(int type, int NB) const { return tiled && tile_of[type][kes::log2_nb(NB)] >= 0; }
+  int own_type() const { return opts.precision == KES_PREC_FP32 ? kes::kTileF32 : kes::kTileF64; }
   // the resident filter (kernels_resident.cu): its plan and the blocks' column ranges, where the
   // matrix is small enough and no launch shape was asked for
   kes::ResidentPlan resident;

@@ -147,8 +147,10 @@ struct TileStep {
   int waits = -1;          // polls of the kernel's waits before they give up, -1: the default
 };
 void launch_tile_step(const TileStep& p, cudaStream_t st);
-// Stages of a tile set's ring that fit a block's shared memory (2 or more: it can run).
+// Stages of a tile set's ring that fit a block's shared memory (2 or more: it can run), and the warps that have
+// rows of that many stages' tiles to add up at a time.
 int tile_stages(int R, int max_xrows, int max_w, int max_head, int row_bytes, int value_bytes, int NB, bool ho);
+int tile_busy_warps(int R, int stages, int value_bytes, int NB);
 // Step values in the order of the tiles (q64 / q32, either may be null), see launch_scale_values.
 struct SellDev;
 void launch_scale_tiles(const SellDev& A, const int4* slice_rec, const int32_t* pat, int n_sm, cudaStream_t st,
