@@ -83,20 +83,25 @@ bool staged_width(const kes_ctx* c, int type, int NB, int cpt) {
   return c->has_tiles(type, NB) && !(type == kTileF32 && too_narrow(c, NB, cpt));
 }
 
-// Whether a staged context runs this filter with the register-staged block kernel all the same:
+// Whether a filter whose width is staged runs with the register-staged block kernel all the same:
 // eight FP32 columns that each add to several weight tables. The staged step keeps one table's
 // accumulators in its stages; the others' 1 KB a row of 16 is latency that its 16 computing warps
-// do not hide (96^3 cells, us a step: 2 tables 41.6 against 43.9 staged, 4 tables 53.9 against
-// 64.5; with one 35.1 against 33.1, and narrower blocks and FP64 are faster staged with 4, too).
+// do not hide (us a step, launch shape / staged, 15 entries a row: 64 thousand rows, 2 tables 5.2 / 5.5, 4 tables 6.4 /
+// 7.3; 96^3 cells 41.6 / 43.9 and 53.9 / 64.5, with one table 35.1 / 33.1; narrower blocks and FP64 are faster
+// staged with 4, too). With fewer rows the blocks' share is small enough (47 thousand rows: 5.1 / 4.8 and 6.2 / 6.2;
+// 16 thousand: 4.1 / 3.0 and 4.8 / 3.6).
+constexpr int64_t kManyTablesRows = 56 * 1024;
 bool many_tables(const kes_ctx* c, int NB, bool fp64, int cpt, bool x2) {
-  return staged_width(c, kTileF32, 8, 0) && !fp64 && !x2 && NB == 8 && cpt == 0 && c->F > 1 &&
-         c->opts.stepper == KES_STEPPER_LEAPFROG;
+  return !fp64 && !x2 && NB == 8 && cpt == 0 && c->F > 1 && c->n_pad >= kManyTablesRows &&
+         c->opts.stepper == KES_STEPPER_LEAPFROG && staged_width(c, kTileF32, 8, 0);
 }
 // The kernel of a filter that does not run as the resident one.
 bool staged_filter(const kes_ctx* c, int NB, bool fp64, int cpt, bool x2) {
   return staged_width(c, x2 ? kTileX2 : fp64 ? kTileF64 : kTileF32, NB, cpt) && !many_tables(c, NB, fp64, cpt, x2);
 }
-constexpr int kManyTablesShape = 13;  // the shape that the autotuner picks for it on the meshes at hand
+// Their launch shape: fixed, since these contexts time no shapes (within 6% of the fastest of all shapes over 47 thousand
+// to 1 million rows of 3 to 27 entries, mostly within 2%).
+constexpr int kManyTablesShape = 13;
 
 // Issues the fused steps of one filter application of an NB-column block on the context
 // stream: stage_in -> stage_out (cpt = 0: F filtered blocks, every column with every
@@ -235,16 +240,25 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
   return g_launches - before;
 }
 
-// Whether a filter application runs as one resident kernel: it fits, and a block has few enough
-// stored entries that 16 SMs a column beat a chain of launches over all of them. In FP64 the 16
-// SMs' FP64 pipes set the line (us a step, resident / staged: 3,360 entries a block, 16^3 cells,
-// 1.6 / 2.7; 7,168, 128^2 cells, 2.4 / 2.3; 11,520, 24^3 cells, 3.5 / 2.7). In FP32 shared memory
-// does (11,520: 1.4 / 2.3; 20,640, 29^3 cells: 2.2 / 2.6), but eight columns of that size no
-// longer run at once (3,584, 64^2 cells: 0.8 / 2.4; 11,520: 2.8 / 2.6).
+// Whether a filter application runs as one resident kernel: it fits, and a block has little enough to do that 16 SMs a
+// column beat a chain of launches over all of them. What a block does in a step is its stored entries, its rows,
+// and its rows once more for each weight table besides the first. In FP64 the 16 SMs' FP64 pipes set the line (us a
+// step, resident / staged: 3,360 entries a block, 16^3 cells, 1.6 / 2.7; 7,168, 128^2 cells, 2.4 / 2.3; 11,520, 24^3
+// cells, 3.5 / 2.7; with 8 tables 2,812 entries and 937 rows 2.6 / 2.9, 4,128 and 1,376 4.1 / 3.5). In FP32 shared
+// memory does (11,520: 1.4 / 2.3; 20,640, 29^3 cells: 2.2 / 2.6), but eight columns of that size no longer run at once
+// (3,584, 64^2 cells: 0.8 / 2.4; 11,520: 2.8 / 2.6). Where the alternative is a launch shape (narrow rows, see
+// too_narrow) the rows decide as much (resident / shape: 1 column, 8,437 entries and 2,812 rows 2.1 / 2.3, with 4
+// tables 2.8 / 2.4; 12,187 and 4,062 2.5 / 2.1; 8 columns, 4,128 and 1,376 2.6 / 2.5; 5,625 and 1,875 2.8 / 2.4).
 bool resident_filter(const kes_ctx* c, int NB, bool fp64, int cpt, int steps, bool x2) {
   if (x2 || c->opts.stepper != KES_STEPPER_LEAPFROG || !c->resident_range) return false;
-  if (c->resident.entries > (fp64 || NB == 8 ? 7000 : 24000)) return false;
-  return resident_fits(c->resident, fp64, cpt ? 1 : c->F, c->n_mesh(), steps);
+  const int tables = cpt ? 1 : c->F;
+  const int64_t entries = c->resident.entries, rows = static_cast<int64_t>(c->resident.slices) * kSliceC;
+  if (entries > (fp64 || NB == 8 ? 7000 : 24000)) return false;
+  if (fp64 && NB == 1 && 10 * entries + 12 * rows * (tables - 1) > 110000) return false;
+  if (!fp64 && entries <= 8 * rows && !staged_width(c, kTileF32, NB, cpt) &&
+      10 * entries + 40 * rows + 9 * rows * (tables - 1) > (NB <= 2 ? 260000 : NB == 4 ? 340000 : 110000))
+    return false;
+  return resident_fits(c->resident, fp64, tables, c->n_mesh(), steps);
 }
 
 // The FP64 step values in the order that the kernels of a width read.
@@ -973,7 +987,7 @@ kes_status set_weights_impl(kes_ctx* c, int32_t F, const double* alpha, const do
     }
     KES_CUDA(cudaMemcpyAsync(c->tau2m64, t2m.data(), c->n_pad * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     // the register-staged block kernel's values, where a filter may take it (many_tables)
-    if (!c->step32 && c->opts.precision == KES_PREC_FP32 && c->NBcap == 8 && F > 1 &&
+    if (!c->step32 && c->opts.precision == KES_PREC_FP32 && c->NBcap == 8 && F > 1 && c->n_pad >= kManyTablesRows &&
         c->opts.stepper == KES_STEPPER_LEAPFROG)
       c->step32 = c->dzero_n<float>(c->nnz_pad);
     // step values A = -tau^2 M^{-1} S (the FP32 ones rounded once from the FP64 product)

@@ -93,33 +93,39 @@ def test_staged_columns_equal_the_launch_shapes(b, F):
 
 
 @pytest.mark.parametrize("use_graph", [True, False])
+@pytest.mark.parametrize("cells,kernel", [((43, 31, 29), "STAGED"), ((53, 43, 39), "SHAPES")])
 @pytest.mark.parametrize("b", [5, 8])
-def test_eight_columns_with_several_tables(b, use_graph):
-    """Eight FP32 columns leave the staged steps for several tables, in one context that goes from one table to
-    several and back with another time step each time."""
-    p = box_grid((53, 43, 39))
+def test_eight_columns_with_several_tables(b, cells, kernel, use_graph):
+    """Eight FP32 columns leave the staged steps for several tables from 56 thousand rows on (83 thousand here), in
+    one context that goes from one table to several and back with another time step each time."""
+    p = box_grid(cells)
     got, ref = [], []
     for out, autotune in ((got, True), (ref, False)):
         with K.Context(p, block_b=b, precision="fp32", autotune=autotune, use_graph=use_graph) as c:
             for F, tau in ((1, 0.004), (4, 0.003), (2, 0.0045), (1, 0.0035)):
                 out.append(_apply(c, p.n, b, F, 8, tau))
+    want = {1: K.KES_KERNEL_STAGED, 2: getattr(K, f"KES_KERNEL_{kernel}"), 4: getattr(K, f"KES_KERNEL_{kernel}")}
     for (a, ka), (r, _), F in zip(got, ref, (1, 4, 2, 1)):
         np.testing.assert_array_equal(a, r)
-        assert ka == (K.KES_KERNEL_STAGED if F == 1 else K.KES_KERNEL_SHAPES)
+        assert ka == want[F]
 
 
 # stored entries a block: a matrix of s slices with w entries a row has ceil(s / 16) * 32 w
 @pytest.mark.parametrize("precision,b,F,n,reach,kernel", [
     ("fp64", 1, 1, 32 * 16 * 14, 7, "RESIDENT"),             # 6,720 entries (the limit is 7,000),
     ("fp64", 1, 1, 32 * 16 * 15, 7, "STAGED"),               # 7,200
-    ("fp64", 1, 4, 32 * 16 * 14, 7, "RESIDENT"),
+    ("fp64", 1, 4, 32 * 16 * 14, 7, "RESIDENT"),             # 6,720 and 448 rows for each further table,
+    ("fp64", 1, 8, 32 * 16 * 40, 2, "STAGED"),               # 6,400 and 1,280 for each of seven
     ("fp64", 8, 2, 32 * 16 * 14, 7, "RESIDENT"),
     ("fp32", 1, 1, 32 * 16 * 50 - 7, 7, "RESIDENT"),         # 24,000
     ("fp32", 1, 1, 32 * 16 * 51, 7, "STAGED"),               # 24,480
     ("fp32", 4, 4, 32 * 16 * 50, 7, "RESIDENT"),
     ("fp32", 8, 1, 32 * 16 * 14, 7, "RESIDENT"),
-    ("fp32", 8, 1, 32 * 16 * 15, 7, "STAGED"),
+    ("fp32", 8, 2, 32 * 16 * 15, 7, "STAGED"),
     # five entries a row: from 20,480 rows on the alternative is a launch shape
+    ("fp32", 1, 1, 32 * 16 * 78, 2, "RESIDENT"),             # 12,480 entries and 2,496 rows,
+    ("fp32", 1, 8, 32 * 16 * 78, 2, "SHAPES"),               # with seven further tables,
+    ("fp32", 8, 1, 32 * 16 * 42, 2, "SHAPES"),               # 6,720 and 1,344 in eight columns
     ("fp32", 2, 1, 32 * 2500, 2, "SHAPES"),
     ("fp32", 1, 1, 32 * 8191, 2, "SHAPES"),                  # one column up to 262,144 rows
     ("fp32", 1, 1, 32 * 8192, 2, "STAGED"),
