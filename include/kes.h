@@ -80,9 +80,10 @@ typedef struct kes_opts {
                           the block size of kes_block_krylov_solve), 1..8; blocks of 2, 4 or 8 columns run
                           as one SpMM step (row-major state), other sizes are padded to the next of them */
   int32_t autotune;    /* 1: the staged step kernels where the matrix allows them (every tile of rows gathers from a few
-                          contiguous runs of rows that fit in shared memory; needs compact_cols), else kes_create
-                          times every launch shape of the step kernels on this matrix and keeps the fastest; 0: the
-                          shape step_variant / blk_variant. Results do not depend on the choice */
+                          contiguous runs of rows, enough of which fit in shared memory; needs compact_cols) and they
+                          are the faster ones, else a launch shape of the register-staged step kernels: a fixed one
+                          for narrow rows, else kes_create times every shape on this matrix and keeps the fastest. 0:
+                          the shape step_variant / blk_variant. Results do not depend on the choice */
   int32_t step_variant; /* launch shape used when autotune is 0 (0 .. number of shapes - 1) */
   void* stream;        /* cudaStream_t for every launch; NULL: the context creates its own non-blocking stream */
   /* Optional device allocator (e.g. a framework's caching allocator). Both NULL: cudaMalloc / cudaFree. */

@@ -93,14 +93,14 @@ bool staged_width(const kes_ctx* c, int type, int NB, int cpt) {
 constexpr int64_t kManyTablesRows = 56 * 1024;
 bool many_tables(const kes_ctx* c, int NB, bool fp64, int cpt, bool x2) {
   return !fp64 && !x2 && NB == 8 && cpt == 0 && c->F > 1 && c->n_pad >= kManyTablesRows &&
-         c->opts.stepper == KES_STEPPER_LEAPFROG && staged_width(c, kTileF32, 8, 0);
+         c->opts.stepper == KES_STEPPER_LEAPFROG && c->has_tiles(kTileF32, 8);
 }
 // The kernel of a filter that does not run as the resident one.
 bool staged_filter(const kes_ctx* c, int NB, bool fp64, int cpt, bool x2) {
   return staged_width(c, x2 ? kTileX2 : fp64 ? kTileF64 : kTileF32, NB, cpt) && !many_tables(c, NB, fp64, cpt, x2);
 }
-// Their launch shape: fixed, since these contexts time no shapes (within 6% of the fastest of all shapes over 47 thousand
-// to 1 million rows of 3 to 27 entries, mostly within 2%).
+// Their launch shape: fixed, since contexts with tiles time no shapes for it (within 6% of the fastest of all shapes over
+// 47 thousand to 1 million rows of 3 to 27 entries, mostly within 2%).
 constexpr int kManyTablesShape = 13;
 
 // Issues the fused steps of one filter application of an NB-column block on the context
@@ -641,6 +641,7 @@ void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, co
   if (!c->tiled) return;
   c->nnz_q = lay.n_values;
   c->narrow = fp32 && !ho && lay.n_values <= 8 * c->n_pad;
+  for (int NB = 1; NB <= c->NBcap; NB *= 2) c->narrow = c->narrow && c->has_tiles(kTileF32, NB);
   c->shapes = false;
   for (int NB = 1; NB <= c->NBcap; NB *= 2)
     c->shapes = c->shapes || !staged_width(c, c->own_type(), NB, 0) || (NB > 1 && !staged_width(c, c->own_type(), NB, 1));
@@ -915,7 +916,16 @@ kes_status create_impl(kes_ctx** out, int32_t nm, const int64_t* n, const int64_
     c->cfg.variant_blk = c->opts.blk_variant;
     c->cfg.grid_blk =
         n_sm * blk_blocks_per_sm(fp32, c->NBcap > 1 ? c->NBcap : 2, c->opts.blk_variant, c->cfg.block_step);
-    if (c->opts.autotune && c->shapes) tune_steps(c);
+    if (c->narrow && c->shapes) {
+      // Narrow rows alone bring the shapes in: they are not timed (their steps are so short that the timing picks
+      // by chance: up to 20% slower than these, which are within 8% and 11% of the fastest shape, 1% and 2% on
+      // average, over 22 to 450 thousand rows of 3 to 7 entries, 1 to 8 columns, 1 and 4 tables).
+      select_variant(c, 4);
+      c->cfg.variant_blk = 12;
+      c->cfg.grid_blk = n_sm * blk_blocks_per_sm(true, c->NBcap > 1 ? c->NBcap : 2, 12, c->cfg.block_step);
+    } else if (c->opts.autotune && c->shapes) {
+      tune_steps(c);
+    }
     c->sync();
     c->stats.bytes_per_step = kes_step_bytes(c, 1, 1);
     shape_stats(c);
