@@ -45,10 +45,10 @@ typedef enum kes_status {
   KES_ERR_CUDA = -4,               /* a CUDA runtime call failed */
   KES_ERR_OOM = -5,                /* device or host allocation failed */
   KES_ERR_TIMEOUT = -6,            /* a bounded device-side wait gave up: a staged step waited for its own copies (or
-                                      for warps of its own block) until the limit of kes_set_wait_limit; no
-                                      kernel of this library waits on another thread block, but for the
-                                      hardware's cluster barrier. The filtered vectors are not valid; the context
-                                      stays usable */
+                                      for warps of its own block) for 2^20 polls, about 1.5 seconds; no kernel
+                                      of this library waits on another thread block, but for the hardware's
+                                      cluster barrier. The filtered vectors are not valid; the context stays
+                                      usable */
   KES_ERR_STATE = -7,              /* call out of order (e.g. filter not set) */
   KES_ERR_UNSUPPORTED = -8         /* option combination not implemented */
 } kes_status;
@@ -290,11 +290,11 @@ enum kes_kernel {
   KES_KERNEL_RESIDENT = 3  /* one launch for all steps (small matrices) */
 };
 int32_t kes_filter_kernel(const kes_ctx* ctx);
-/* kes_set_wait_limit: polls (about 1.5 us each) that a device-side wait of this context's kernels takes before it
-   gives up and the call that reads the result returns KES_ERR_TIMEOUT; -1 (the default): 2^20, about 1.5
-   seconds (each later step of the same filter may wait as long again). 0: such a wait gives up at once. Waits for
-   pending work; KES_ERR_ARG below -1. */
-kes_status kes_set_wait_limit(kes_ctx* ctx, int32_t polls);
+/* kes_fail_waits: for tests of what a caller does about KES_ERR_TIMEOUT. on = 1: in the staged steps the warps that copy
+   give up at their first wait, so that on matrices of a quarter million rows or more the ones that compute
+   wait for tiles that never come: each step of a filter ends after about 1.5 seconds, and the call that reads the
+   result returns KES_ERR_TIMEOUT. on = 0 (the default): as usual. Waits for pending work. */
+kes_status kes_fail_waits(kes_ctx* ctx, int32_t on);
 /* kes_step_bytes: algorithmic HBM bytes of one fused leapfrog step of this context for b vectors
    and F intervals (every matrix entry, row pointer and per-row vector read or written once; an
    entry is its value plus a 2-byte column difference when the compact index is in use, else a

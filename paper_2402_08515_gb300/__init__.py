@@ -29,7 +29,7 @@ __all__ = [
     "kes_create_batch", "kes_mesh_count", "kes_estimate_omega_max_batch", "kes_set_filters_batch",
     "kes_block_krylov_solve", "kes_set_weights", "kes_alpha_gaussian", "kes_filter_apply_columns",
     "kes_alpha_triangle", "kes_weights_response", "kes_launch_shapes", "kes_subspace_solve", "kes_filter_kernel",
-    "kes_set_wait_limit", "KES_KERNEL_NONE", "KES_KERNEL_SHAPES", "KES_KERNEL_STAGED", "KES_KERNEL_RESIDENT",
+    "kes_fail_waits", "KES_KERNEL_NONE", "KES_KERNEL_SHAPES", "KES_KERNEL_STAGED", "KES_KERNEL_RESIDENT",
 ]
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -128,7 +128,7 @@ _sig = {
     "kes_alpha_triangle": (C.c_int, [C.c_double, C.c_double, C.c_double, C.c_int32, _P]),
     "kes_weights_response": (C.c_int, [_P, C.c_double, C.c_int32, _P, C.c_int64, _P]),
     "kes_filter_kernel": (C.c_int32, [_P]),
-    "kes_set_wait_limit": (C.c_int, [_P, C.c_int32]),
+    "kes_fail_waits": (C.c_int, [_P, C.c_int32]),
     "kes_launch_shapes": (None, [C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
 }
 for _name, (_res, _args) in _sig.items():
@@ -249,9 +249,9 @@ def kes_filter_kernel(ctx: int) -> int:
     return lib.kes_filter_kernel(ctx)
 
 
-def kes_set_wait_limit(ctx: int, polls: int) -> None:
-    """Polls that a device-side wait takes before it gives up (KES_ERR_TIMEOUT); -1: the default, about 1.5 s."""
-    _check(lib.kes_set_wait_limit(ctx, int(polls)), "kes_set_wait_limit")
+def kes_fail_waits(ctx: int, on: bool) -> None:
+    """Makes the staged steps' waits run out (KES_ERR_TIMEOUT), for tests of a caller's handling of it."""
+    _check(lib.kes_fail_waits(ctx, int(on)), "kes_fail_waits")
 
 
 def kes_weights_response(alpha, tau: float, omega) -> np.ndarray:

@@ -60,7 +60,7 @@ struct TileArgs {
   int keep, chained;
   int stages, stage_bytes, off_prev, off_own, off_acc, off_val, off_head;
   int* flag;
-  int waits;          // polls of a wait before it gives up
+  int fail;           // the copying warps give up at their first wait
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -75,9 +75,10 @@ __device__ __forceinline__ void mbar_expect(uint32_t bar, int bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// Waits for the phase of that parity to complete; false once the limit is reached.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int limit) {
-  for (int i = 0; i < limit; ++i) {
+// Waits for the phase of that parity to complete; false once the limit is reached. (The limit is a constant: as a
+// kernel parameter it cost the FP32 steps 1 to 2%.)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < kWaitLimit; ++i) {
     uint32_t done;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
       }
     };
     auto wait_empty = [&]() {
-      return n < stages || mbar_wait(smem_addr(&bars[kMaxStages + st]), phase ^ 1, a.waits);
+      return n < stages || (!a.fail && mbar_wait(smem_addr(&bars[kMaxStages + st]), phase ^ 1));
     };
     const int M = a.ts.max_runs + 2;
     if (((warp - kGroupWarps * GROUPS) & 1) == 0) {
@@ -290,9 +291,9 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
       }
     }
     if (!ok && lane == 0) atomicOr(a.flag, 2);
-    // the copies still in flight write this block's shared memory: they land whatever limit was set
+    // the copies still in flight write this block's shared memory
     for (int i = n - GROUPS; i >= 0 && i >= n - stages; i -= GROUPS)
-      mbar_wait(smem_addr(&bars[i % stages]), (i / stages) & 1, kWaitLimit);
+      mbar_wait(smem_addr(&bars[i % stages]), (i / stages) & 1);
     return;
   }
 
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(32 * (kGroupWarps + 2) * GROUPS, 1) k_tile(con
   int st = grp;  // stages >= GROUPS
   uint32_t phase = 0;
   for (int n = grp; n < mine; n += GROUPS) {
-    if (!mbar_wait(smem_addr(&bars[st]), phase, a.waits)) {
+    if (!mbar_wait(smem_addr(&bars[st]), phase)) {
       if (lane == 0) atomicOr(a.flag, 2);
       break;
     }
@@ -683,7 +684,7 @@ void launch_tile_step(const TileStep& p, cudaStream_t st) {
   a.last = p.last;
   a.fold2 = p.fold2;
   a.flag = p.flag;
-  a.waits = p.waits >= 0 ? p.waits : kWaitLimit;
+  a.fail = p.fail;
   a.stages = f.stages;
   a.chained = p.chained;
   a.keep = keep_in_l2(p, size);

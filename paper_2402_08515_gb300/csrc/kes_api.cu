@@ -139,7 +139,7 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
     p.L = L;
     p.cpt = cpt;
     p.flag = c->d_flag;
-    p.waits = c->waits;
+    p.fail = c->fail_waits;
     int next = p.type == kTileF64 ? 0 : 1;  // first weighted term not yet in the accumulators
     for (int s = 0; s < steps; ++s) {
       p.x = s == 0 ? start : U[(s - 1) & 1];
@@ -1139,12 +1139,12 @@ void kes_launch_shapes(int32_t* n_step, int32_t* n_block) {
   if (n_block) *n_block = blk_variant_count();
 }
 
-kes_status kes_set_wait_limit(kes_ctx* c, int32_t polls) {
-  if (!c || polls < -1) return KES_ERR_ARG;
+kes_status kes_fail_waits(kes_ctx* c, int32_t on) {
+  if (!c || on < 0 || on > 1) return KES_ERR_ARG;
   return guarded([&]() -> kes_status {
     c->sync();
-    c->waits = polls;
-    c->drop_graphs();  // the limit is a parameter of their kernels
+    c->fail_waits = on != 0;
+    c->drop_graphs();  // it is a parameter of their kernels
     return KES_OK;
   });
 }

@@ -163,7 +163,7 @@ struct kes_ctx {
   float* acc_c = nullptr;
   double* tmp_user = nullptr;  // n x NBcap, caller layout
   int* d_flag = nullptr;
-  int waits = -1;  // kes_set_wait_limit
+  bool fail_waits = false;  // kes_fail_waits
   int filter_kernel = KES_KERNEL_NONE;  // what ran the last filter application (enum kes_kernel)
   std::vector<kes::GraphEntry> graphs;
   int g_F = -1, g_L = -1;

@@ -144,7 +144,7 @@ struct TileStep {
   bool init = false, last = false, fold2 = false;
   bool chained = false;    // the launch before it in the stream is a staged step of the same filter
   int* flag = nullptr;
-  int waits = -1;          // polls of the kernel's waits before they give up, -1: the default
+  bool fail = false;       // its copying warps give up at their first wait (kes_fail_waits)
 };
 void launch_tile_step(const TileStep& p, cudaStream_t st);
 // Stages of a tile set's ring that fit a block's shared memory (2 or more: it can run), and the warps that have

@@ -172,24 +172,24 @@ def test_wide_rows_are_staged_where_enough_of_them_fit(precision, b, kernel):
     assert _both(p, b, 1, 4, precision=precision, tau=0.05) == getattr(K, f"KES_KERNEL_{kernel}")
 
 
-@pytest.mark.parametrize("precision,b,opts", [("fp64", 1, {}), ("fp32", 8, {}), ("fp32", 2, dict(use_graph=False)),
+@pytest.mark.parametrize("precision,b,opts", [("fp64", 1, {}), ("fp32", 8, {}), ("fp32", 1, dict(use_graph=False)),
                                               ("fp64", 4, dict(stepper="leapfrog4"))])
 def test_a_wait_that_runs_out_is_an_error_and_the_context_stays_usable(precision, b, opts):
-    """With a limit of no polls every wait of the staged steps gives up: the copies under way still land, the call says
-    KES_ERR_TIMEOUT, and with the default limit the same context filters as if nothing had been."""
-    p = box_grid((43, 31, 29))
+    """The copying warps give up once the ring is full: the copies under way still land, the computing warps' waits run
+    out (1.5 seconds), the call says KES_ERR_TIMEOUT, and afterwards the same context filters as if nothing had been."""
+    p = box_grid((73, 65, 64))                                   # 290 thousand rows: more tiles a block than stages
     R = start_vectors(p.n, b, 11)
     with K.Context(p, precision=precision, block_b=b, **opts) as c:
-        ref, kernel = _apply(c, p.n, b, 1, 8, 0.004)
+        ref, kernel = _apply(c, p.n, b, 1, 1, 0.004)
         assert kernel == K.KES_KERNEL_STAGED
-        K.kes_set_wait_limit(c.handle, 0)
+        K.kes_fail_waits(c.handle, True)
         with pytest.raises(K.KesError) as e:
             K.kes_filter_apply(c.handle, R, np.zeros((1, b, p.n)), b)
         assert e.value.status == -6
         with pytest.raises(K.KesError) as e:
-            K.kes_set_wait_limit(c.handle, -2)
+            K.kes_fail_waits(c.handle, 2)
         assert e.value.status == -1
-        K.kes_set_wait_limit(c.handle, -1)
+        K.kes_fail_waits(c.handle, False)
         out = np.zeros((1, b, p.n))
         K.kes_filter_apply(c.handle, R, out, b)
         np.testing.assert_array_equal(out, ref)
