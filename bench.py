@@ -204,13 +204,25 @@ def kernel_source_hash(src: str = STEP_KERNEL_SRC) -> str:
     return hashlib.sha256("\n".join(code).encode()).hexdigest()[:16]
 
 
-def step_bytes(K, h, problems, precision, b, F, L, staged) -> int:
-    """Algorithmic bytes of an average step. The staged kernels read no row pointers, and no columns on tensor grids
-    (rows of a tile are shifted copies of one another) and 2-byte places elsewhere; the launch shapes read what
-    kes_step_bytes counts."""
-    if not staged:
-        return K.kes_step_bytes(h, b, F)
+def filter_kernel(K, h, precision, b) -> str:
+    """The kernel that ran the context's last filter application of b columns."""
+    T, nb = ("double", "float")[precision == "fp32"], 1 if b == 1 else 2 if b == 2 else 4 if b <= 4 else 8
+    shape = ("k_step_f64", "k_step_f32")[precision == "fp32"] if nb == 1 else f"k_step_blk<{T},{nb}>"
+    return {K.KES_KERNEL_STAGED: f"k_tile<{T},{nb}>", K.KES_KERNEL_RESIDENT: f"k_resident<{T}>",
+            K.KES_KERNEL_SHAPES: shape}[K.kes_filter_kernel(h)]
+
+
+def step_bytes(K, h, problems, precision, b, F, L) -> int:
+    """Algorithmic HBM bytes of an average step of the context's last filter application (b columns, F tables, L steps).
+    The staged kernels read no row pointers, and no columns on tensor grids (rows of a tile are shifted copies of one
+    another) and 2-byte places elsewhere; the launch shapes read what kes_step_bytes counts; the resident filter reads
+    S and its columns, the start block and nothing more, and writes the result, once for all steps."""
     n, nnz = sum(p.n for p in problems), sum(p.nnz for p in problems)
+    kernel = K.kes_filter_kernel(h)
+    if kernel == K.KES_KERNEL_RESIDENT:
+        return (12 * nnz + 8 * n * b * (1 + F)) // L
+    if kernel != K.KES_KERNEL_STAGED:
+        return K.kes_step_bytes(h, b, F)
     size = 8 if precision == "fp64" else 4
     nxt, adds = (0 if size == 8 else 1), 0   # the steps that add weighted terms: every third and the last
     for s in range(L):
@@ -521,12 +533,12 @@ def batch_filter_measurement(dev, stream, reps: int = 3) -> dict:
                 K.kes_filter_apply(h, R, res, wl.b)
             st = K.kes_get_stats(h)
             step_us = 1e3 * st["filter_ms"] / max(st["filter_steps"], 1)
-            nbytes = step_bytes(K, h, problems, wl.precision, wl.b, F, wl.L, st["blk_variant"] == -1)
+            nbytes = step_bytes(K, h, problems, wl.precision, wl.b, F, wl.L)
             gbs = nbytes / (step_us / 1e6) / 1e9
-            out[f"F{F}"] = {"step_us": step_us, "algorithmic_bytes_per_step": nbytes, "achieved_gbs": gbs,
+            out[f"F{F}"] = {"kernel": filter_kernel(K, h, wl.precision, wl.b), "step_us": step_us, "algorithmic_bytes_per_step": nbytes, "achieved_gbs": gbs,
                             "frac": gbs / peak, "gdof_steps_per_s": n * wl.b / (step_us / 1e6) / 1e9,
                             "finite": bool(torch.isfinite(res).all())}
-        out["kernel"] = "k_tile<float,8>" if st["blk_variant"] == -1 else "k_step_blk<float,8>"
+        out["kernel"] = out["F1"]["kernel"]
         out["blk_variant"] = st["blk_variant"]
         out["timing"] = f"{reps} filter applications of {wl.L} steps, CUDA events on the library stream, after one warm"
     return out
@@ -649,11 +661,11 @@ def run_kes(args):
 
     # roofline of the fused step kernel, timed by the library's CUDA events on its stream
     step_ms = stats["filter_ms"] / max(stats["filter_steps"], 1)
-    staged = stats["step_variant"] == -1
-    bytes_step = step_bytes(K, h, problems, wl.precision, b, 1, wl.L, staged)
+    kernel = filter_kernel(K, h, wl.precision, b)
+    bytes_step = step_bytes(K, h, problems, wl.precision, b, 1, wl.L)
     achieved = bytes_step / (step_ms / 1e3) / 1e9
     peak, peak_src = load_peak()
-    traffic = profiled_traffic(args.workload, STEP_KERNEL_SRC if b == 1 else BLOCK_KERNEL_SRC) if staged else None
+    traffic = profiled_traffic(args.workload) if kernel.startswith("k_tile") else None
 
     # several intervals from one trajectory: the same block filtered with F weight tables
     multi = None
@@ -668,8 +680,8 @@ def run_kes(args):
             K.kes_filter_apply(h, R0_dev, out, b)
         st = K.kes_get_stats(h)
         fms = st["filter_ms"] / reps
-        bF = step_bytes(K, h, problems, wl.precision, b, F, wl.L, staged)
-        multi = {"F": F, "b": b, "L": wl.L, "ms_per_filter": fms,
+        bF = step_bytes(K, h, problems, wl.precision, b, F, wl.L)
+        multi = {"F": F, "b": b, "L": wl.L, "kernel": filter_kernel(K, h, wl.precision, b), "ms_per_filter": fms,
                  "value": n * b * wl.L / (fms / 1e3) / 1e9, "unit": METRIC,
                  "step_us": 1e3 * fms / wl.L, "achieved_gbs": bF / (fms / wl.L / 1e3) / 1e9,
                  "algorithmic_bytes_per_step": bF}
@@ -784,9 +796,7 @@ def run_kes(args):
                    "l2": "inputs larger than L2 (matrix > 129 MB)"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
-                     "kernel": f"k_tile<{'double' if wl.precision == 'fp64' else 'float'},{b}>" if staged
-                     else ("k_step_f64" if wl.precision == "fp64" else "k_step_f32") if b == 1
-                     else ("k_step_blk<double>" if wl.precision == "fp64" else "k_step_blk<float>"),
+                     "kernel": kernel,
                      "step_variant": stats["step_variant"] if b == 1 else stats["blk_variant"],
                      "step_grid": stats["step_grid"] if b == 1 else stats["blk_grid"],
                      "step_us": step_ms * 1e3, "algorithmic_bytes_per_step": bytes_step},

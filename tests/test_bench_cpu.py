@@ -76,3 +76,24 @@ def test_time_to_solution_forms_are_well_formed():
         assert prec in ("fp64", "fp32") and b in (1, 8) and 0 < frac <= 1.0 and extra >= 0
         assert (sweeps > 0) == (prec == "fp32")        # the FP32 forms are refined, FP64 ones not
         assert rprec in (0, 1) and ("x2" in name) == (rprec == 1)
+
+
+def test_step_bytes_and_kernel_name_follow_the_kernel_that_ran():
+    # the staged steps, the launch shapes and the resident filter read different bytes: both come from what the library
+    # says it ran, not from the launch shape in its statistics (which does not tell them apart)
+    from types import SimpleNamespace
+
+    def K(kernel):
+        return SimpleNamespace(KES_KERNEL_SHAPES=1, KES_KERNEL_STAGED=2, KES_KERNEL_RESIDENT=3,
+                               kes_filter_kernel=lambda h: kernel, kes_step_bytes=lambda h, b, F: 12345)
+    p = square_grid(24)
+    n, nnz = p.n, p.nnz
+    assert "extent" in p.meta
+    L, F, b = 9, 2, 8                                            # FP32: three of nine steps add weighted terms
+    names = {(1, 1): "k_step_f32", (1, 8): "k_step_blk<float,8>", (2, 5): "k_tile<float,8>", (3, 8): "k_resident<float>"}
+    for (kernel, cols), name in names.items():
+        assert bench.filter_kernel(K(kernel), None, "fp32", cols) == name
+    assert bench.filter_kernel(K(2), None, "fp64", 3) == "k_tile<double,4>"
+    assert bench.step_bytes(K(1), None, [p], "fp32", b, F, L) == 12345
+    assert bench.step_bytes(K(2), None, [p], "fp32", b, F, L) == 4 * nnz + n * b * 12 + n * b * 16 * F * 3 // 9
+    assert bench.step_bytes(K(3), None, [p], "fp32", b, F, L) == (12 * nnz + 8 * n * b * 3) // 9
