@@ -436,8 +436,9 @@ kes_status kes_filter_apply_noalloc(int64_t n, const int64_t* row_ptr, const int
 /*
  * kes_filter_apply_noalloc_sized -- the same with the number of stored entries given by the caller, who has it on
  * the host (row_ptr stays on the device and is not read there): a matrix of wide rows (48 entries on average or
- * more, from 20,000 rows on) then runs with a kernel made for them, about a fifth to a half faster. The
- * number decides nothing else and need not be exact; -1: not known, as kes_filter_apply_noalloc.
+ * more, from 20,000 rows on) then runs with a kernel made for them, 1.3 to 1.8 times as fast, and a small matrix of
+ * short rows (16 on average or fewer) without blocks for wide ones, 4% faster. The number decides nothing else and
+ * need not be exact; -1: not known, as kes_filter_apply_noalloc.
  */
 kes_status kes_filter_apply_noalloc_sized(int64_t n, int64_t nnz, const int64_t* row_ptr, const int32_t* col,
                                           const double* val, const double* tau2m, const double* alpha, int32_t L,

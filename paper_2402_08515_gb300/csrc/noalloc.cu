@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_step_csr_f64(int64_t n, const i
   if (blockIdx.y > 0 && !chunks) return;
   const int64_t first = row < n ? row_ptr[row] : end, stop = row < n ? row_ptr[row + 1] : end;
   auto stage = [&](int64_t c0, int count) {
-#pragma unroll 8
+#pragma unroll 4
     for (int i = tid; i < count; i += kThreads) {
       s_val[place(i)] = __ldcs(val + c0 + i);
       s_col[place(i)] = __ldcs(col + c0 + i);
@@ -219,12 +219,10 @@ __global__ void __launch_bounds__(256) k_step_csr_wide_f64(int64_t n, const int6
 }
 
 template <bool FIRST, bool LAST>
-cudaError_t launch_step(bool wide, int64_t n, cudaStream_t st, const int64_t* row_ptr, const int32_t* col, const double* val,
-                        const double* tau2m, const double* x, const double* prev, double* out, double* acc,
-                        const double* alpha, int step) {
+cudaError_t launch_step(bool wide, unsigned split, int64_t n, cudaStream_t st, const int64_t* row_ptr,
+                        const int32_t* col, const double* val, const double* tau2m, const double* x,
+                        const double* prev, double* out, double* acc, const double* alpha, int step) {
   const unsigned groups = static_cast<unsigned>((n + kThreads - 1) / kThreads);
-  unsigned split = kMaxSplit;
-  while (split > 1 && groups * split > kBlocks) split /= 2;
   cudaLaunchConfig_t c{};
   c.gridDim = wide ? dim3(static_cast<unsigned>((n * kRowLanes + 255) / 256)) : dim3(groups, split);
   c.blockDim = dim3(wide ? 256 : kThreads);
@@ -279,6 +277,10 @@ extern "C" kes_status kes_filter_apply_noalloc_sized(int64_t n, int64_t nnz, con
   }
   double* U[2] = {state, state + KES_NOALLOC_MAX_N};
   const bool wide = n >= kWideRows && nnz / n >= kWideEntries;
+  // blocks of a group: not where the rows are known to be short on average (the blocks that leave at once cost a small
+  // matrix 4% of a step)
+  unsigned split = nnz >= 0 && nnz <= 16 * n ? 1 : kMaxSplit;
+  while (split > 1 && static_cast<unsigned>((n + kThreads - 1) / kThreads) * split > kBlocks) split /= 2;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   for (int s = 0; s < L; ++s) {
     const bool first = s == 0, last = s == L - 1;
@@ -287,7 +289,7 @@ extern "C" kes_status kes_filter_apply_noalloc_sized(int64_t n, int64_t nnz, con
     double* out = U[s & 1];
     const auto go = first ? (last ? launch_step<true, true> : launch_step<true, false>)
                           : (last ? launch_step<false, true> : launch_step<false, false>);
-    if (go(wide, n, st, row_ptr, col, val, tau2m, x, prev, out, r_out, alpha, s) != cudaSuccess) {
+    if (go(wide, split, n, st, row_ptr, col, val, tau2m, x, prev, out, r_out, alpha, s) != cudaSuccess) {
       cudaGetLastError();
       return KES_ERR_CUDA;
     }
