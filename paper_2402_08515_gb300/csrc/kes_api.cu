@@ -76,7 +76,8 @@ double cfl_bound(const kes_ctx* c) { return c->opts.stepper == KES_STEPPER_LEAPF
 // 300 thousand 4.8 / 4.5, 1 million 16.3 / 12.9). Matrices of up to 20 thousand rows mostly run as the resident filter.
 bool too_narrow(const kes_ctx* c, int NB, int cpt) {
   if (!c->narrow) return false;
-  const int64_t from = cpt > 0 ? 56 * 1024 : 20 * 1024, to = int64_t(1) << (NB == 1 && c->nnz_q > 4 * c->n_pad ? 18 : 19);
+  const int64_t from = cpt > 0 ? 56 * 1024 : 20 * 1024;
+  const int64_t to = int64_t(1) << (NB == 1 && c->nnz_q > 4 * c->n_pad ? 18 : 19);
   return c->n_pad >= from && c->n_pad < to;
 }
 bool staged_width(const kes_ctx* c, int type, int NB, int cpt) {
@@ -124,7 +125,8 @@ int64_t issue_filter_steps(kes_ctx* c, int NB, bool fp64, int cpt, int steps, bo
     p.fold2 = (x2 || fp64) && c->fold64;
     void* start = x2 ? static_cast<void*>(c->U2[2]) : fp64 ? static_cast<void*>(c->stage_in) : c->U32[2];
     void* U[2];
-    for (int j = 0; j < 2; ++j) U[j] = x2 ? static_cast<void*>(c->U2[j]) : fp64 ? static_cast<void*>(c->U64[j]) : c->U32[j];
+    for (int j = 0; j < 2; ++j)
+      U[j] = x2 ? static_cast<void*>(c->U2[j]) : fp64 ? static_cast<void*>(c->U64[j]) : c->U32[j];
     if (x2)
       launch_init_x2(c->stream, c->A, NB, c->stage_in, c->U2[2], c->acc_s, c->acc_c, stride, F, c->alpha64, L, cpt);
     else if (!fp64)
@@ -603,17 +605,28 @@ void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, co
           tried[i] = true;
           ok[i] = build_tiles(in, lay, kTileGroup >> i, built[i]);
         }
-        return ok[i] ? tile_stages(built[i].R, built[i].max_xrows, built[i].max_w, built[i].max_head, size * NB, size, NB, ho)
-                     : 0;
+        const TileHost& t = built[i];
+        return ok[i] ? tile_stages(t.R, t.max_xrows, t.max_w, t.max_head, size * NB, size, NB, ho) : 0;
       };
-      int pick = -1, busy = 0;
+      int pick = -1;
       for (int want = 4; want >= (type == kTileX2 ? 2 : 4) && pick < 0; want -= 2)
         for (int q = 0; q < 4 && pick < 0; ++q)
           if (stages_of(order[q]) >= want) pick = order[q];
-      // the pick may have few rows because the matrix has few; the largest tiles that fit tell
-      for (int i = 0; i < 4 && pick >= 0 && busy == 0; ++i)
-        if (const int stages = stages_of(i); stages >= 4) busy = tile_busy_warps(kTileGroup >> i, stages, size, NB);
-      if (type != kTileX2 && busy < 4) pick = -1;
+      if (type != kTileX2 && pick >= 0) {
+        auto busy = [&](int i) {
+          const int stages = stages_of(i);
+          return stages >= 4 && tile_busy_warps(kTileGroup >> i, stages, size, NB) >= 4;
+        };
+        // The pick may have few rows because the matrix has few: larger tiles tell, too. Twice its rows take at most
+        // twice its runs (with gaps between them staged) and heads; where those fit nothing more is laid out to know.
+        const TileHost& t = built[pick];
+        bool enough = busy(pick);
+        if (!enough && pick > 0 && 2 * t.max_runs <= kMaxRuns)
+          enough = tile_stages(2 * t.R, 2 * (t.max_xrows + 16 * t.max_runs), t.max_w, 2 * t.max_head, size * NB, size,
+                               NB, ho) >= 4;
+        for (int i = 0; i < pick && !enough; ++i) enough = busy(i);
+        if (!enough) pick = -1;
+      }
       c->tile_of[type][log2_nb(NB)] = pick;
       if (type == kTileX2 && pick < 0) {  // the pairs' values have one order for all widths
         for (int& t : c->tile_of[type]) t = -1;
@@ -644,7 +657,7 @@ void plan_tiles(kes_ctx* c, int64_t n_slices, const std::vector<int64_t>& sp, co
   for (int NB = 1; NB <= c->NBcap; NB *= 2) c->narrow = c->narrow && c->has_tiles(kTileF32, NB);
   c->shapes = false;
   for (int NB = 1; NB <= c->NBcap; NB *= 2)
-    c->shapes = c->shapes || !staged_width(c, c->own_type(), NB, 0) || (NB > 1 && !staged_width(c, c->own_type(), NB, 1));
+    c->shapes |= !staged_width(c, c->own_type(), NB, 0) || (NB > 1 && !staged_width(c, c->own_type(), NB, 1));
   c->slice_rec = upload(c, lay.slice_rec);
   c->tile_pat = upload(c, lay.pat);
   c->sync();  // the host vectors go out of scope
@@ -891,7 +904,7 @@ kes_status create_impl(kes_ctx** out, int32_t nm, const int64_t* n, const int64_
     c->tau2m64 = c->dzero_n<double>(np);
     bool own_staged = false;
     for (int NB = 1; NB <= c->NBcap; NB *= 2)
-      own_staged = own_staged || staged_width(c, c->own_type(), NB, 0) || (NB > 1 && staged_width(c, c->own_type(), NB, 1));
+      own_staged |= staged_width(c, c->own_type(), NB, 0) || (NB > 1 && staged_width(c, c->own_type(), NB, 1));
     if (c->opts.precision == KES_PREC_FP32) {
       if (own_staged) c->q32 = c->dzero_n<float>(c->nnz_q);  // zero where a row lacks its pattern's entry
       if (c->shapes) c->step32 = c->dzero_n<float>(c->nnz_pad);
