@@ -296,9 +296,11 @@ int32_t kes_filter_kernel(const kes_ctx* ctx);
    result returns KES_ERR_TIMEOUT. on = 0 (the default): as usual. Waits for pending work. */
 kes_status kes_fail_waits(kes_ctx* ctx, int32_t on);
 /* kes_step_bytes: algorithmic HBM bytes of one fused leapfrog step of this context for b vectors
-   and F intervals (every matrix entry, row pointer and per-row vector read or written once; an
+   and F intervals, as the launch shapes of the register-staged kernels read them (the staged steps read no
+   row pointers, and no columns or 2-byte places, see kes_filter_kernel; a resident filter reads the matrix once
+   for all steps): every matrix entry, row pointer and per-row vector read or written once; an
    entry is its value plus a 2-byte column difference when the compact index is in use, else a
-   4-byte column; the fourth-order stepper adds its stage pass and the read of the stage). The
+   4-byte column; the fourth-order stepper adds its stage pass and the read of the stage. The
    step kernels add the weighted terms of eq. (disc_filtercoeff) to their accumulators every third
    step and at the last (a step holds u_{n-1}, u_n, u_{n+1}), so the accumulator bytes count with
    that share of a filter application of the context's filter length L (the average step). */
@@ -314,7 +316,9 @@ int64_t kes_step_bytes(const kes_ctx* ctx, int32_t b, int32_t F);
  *   b      1 <= b <= opts.block_b; the b vectors share one trajectory (SpMM step)
  * Device pointers: asynchronous on the context stream. Host pointers: the
  * call copies in, runs and copies out before returning.
- * KES_ERR_UNSTABLE if a non-finite value appeared in the state.
+ * KES_ERR_UNSTABLE if a non-finite value appeared in the state (device pointers: from kes_sync). The columns of
+ * the mesh that it appeared in are then no result, and which of their entries are finite depends on the kernel that
+ * ran (kes_filter_kernel); other meshes and other columns are not affected.
  */
 kes_status kes_filter_apply(kes_ctx* ctx, const double* r_in, double* r_out, int32_t b, int32_t mem);
 

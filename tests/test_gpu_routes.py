@@ -193,3 +193,24 @@ def test_a_wait_that_runs_out_is_an_error_and_the_context_stays_usable(precision
         out = np.zeros((1, b, p.n))
         K.kes_filter_apply(c.handle, R, out, b)
         np.testing.assert_array_equal(out, ref)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("kernel", ["RESIDENT", "STAGED", "SHAPES"])
+@pytest.mark.parametrize("b", [1, 3])
+def test_a_value_that_is_not_finite_stays_in_its_mesh_and_column(b, kernel, precision):
+    """An infinite start value is reported, and the other meshes' and the other columns' results are the bits that they
+    are without it (the staged steps hold zeros for couplings that a row lacks, but none out of its mesh)."""
+    p = [square_grid(20), box_grid((9, 8, 7))] if kernel == "RESIDENT" else MATRICES["batch"]()
+    n, n0 = sum(q.n for q in p), p[0].n
+    with K.Context(p, block_b=b, precision=precision, autotune=kernel != "SHAPES") as c:
+        ref, ran = _apply(c, n, b, 1, 6, 0.004)
+        assert ran == getattr(K, f"KES_KERNEL_{kernel}")
+        R, out = start_vectors(n, b, 11), np.zeros((1, b, n))
+        R[b - 1, n0 - 1] = np.inf                                # the last row of the first mesh
+        with pytest.raises(K.KesError) as e:
+            K.kes_filter_apply(c.handle, R, out, b)
+        assert e.value.status == -3
+        assert not np.isfinite(out[0, b - 1, :n0]).all()
+        np.testing.assert_array_equal(out[..., n0:], ref[..., n0:])
+        np.testing.assert_array_equal(out[:, :b - 1], ref[:, :b - 1])
