@@ -189,8 +189,8 @@ __global__ void __launch_bounds__(kThreads, 8) k_step_csr_f64(int64_t n, const i
 
 // The same step for a matrix of wide rows, where the caller says that it is one: eight lanes a row straight from
 // memory, with all of L1 for the gathers and twice the threads that shared memory leaves above (81 entries a row,
-// us a step, shared rows above / this: 50 thousand rows 27.0 / 15.6, 150 thousand 60.2 / 46.6; 121 entries, 300 thousand
-// rows 179.6 / 112.0). The lanes' loop is not unrolled: four entries of a lane at a time lie in other lines than the
+// us a step, shared rows above / this: 50 thousand rows 27.0 / 15.6, 150 thousand 60.2 / 46.6; 121 entries, 300
+// thousand rows 179.6 / 112.0). The lanes' loop is not unrolled: four entries of a lane at a time lie in other lines than the
 // ones at hand, which its neighbours still read (112.0 us against 157.4).
 template <bool FIRST, bool LAST>
 __global__ void __launch_bounds__(256) k_step_csr_wide_f64(int64_t n, const int64_t* __restrict__ row_ptr,
@@ -232,8 +232,8 @@ cudaError_t launch_step(bool wide, unsigned split, int64_t n, cudaStream_t st, c
   at[0].val.programmaticStreamSerializationAllowed = 1;
   c.attrs = at;
   c.numAttrs = FIRST ? 0 : 1;  // the first step follows the caller's own work
-  return cudaLaunchKernelEx(&c, wide ? k_step_csr_wide_f64<FIRST, LAST> : k_step_csr_f64<FIRST, LAST>, n, row_ptr, col, val, tau2m, x, prev, out, acc, alpha,
-                            step);
+  return cudaLaunchKernelEx(&c, wide ? k_step_csr_wide_f64<FIRST, LAST> : k_step_csr_f64<FIRST, LAST>, n, row_ptr,
+                            col, val, tau2m, x, prev, out, acc, alpha, step);
 }
 
 std::mutex g_setup_mu;
