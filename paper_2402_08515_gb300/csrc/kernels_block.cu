@@ -218,8 +218,8 @@ __device__ __forceinline__ void row_sums_pipe(T (&un)[NH], const T* __restrict__
 // The FP64 pipe bounds the FP64 block step (GB300 issues two FP64 operations per clock per
 // SM, all others at 64 times that), so little but the FMAs of the sum may go there: the first
 // weighted term is an FMA onto -0 instead of a product beside an FMA, and the optional 2 u_n of
-// the seed a predicated FMA instead of a select behind one (the sign flip stays an FP64
-// instruction, whatever form it is written in here). 857,375 rows: 63.1 -> 55.3 us per step at 2
+// the seed a predicated FMA instead of a select behind one. (The sign flip of neg() stays an FP64
+// instruction, as -x would be; kernels_tile.cu splits the register pair to have none.) 857,375 rows: 63.1 -> 55.3 us per step at 2
 // columns, 120.0 -> 104.7 us at 4, 207.6 -> 204.9 us at 8 (where the row loads' latency shares the
 // bound).
 __device__ __forceinline__ double neg(double x) {
