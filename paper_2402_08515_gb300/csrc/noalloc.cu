@@ -95,7 +95,10 @@ __device__ __forceinline__ void add_range(double (&s)[4], int k, int ke, const d
     if (k + j < ke) s[j] = fma(s_val[place(k + j)], x[s_col[place(k + j)]], s[j]);
 }
 
-template <bool FIRST, bool LAST>
+// AHEAD: entries of a thread whose copies are under way together. Eight where the rows are short and the grid has
+// no blocks that wait for a place, four elsewhere (us a step, four / eight: 15 entries a row, 29,791 rows 3.72 / 3.67,
+// 64 thousand 6.29 / 6.10, 405 thousand 34.8 / 36.4; 27 entries, 27 thousand rows 7.5 / 7.9).
+template <bool FIRST, bool LAST, int AHEAD>
 __global__ void __launch_bounds__(kThreads, 8) k_step_csr_f64(int64_t n, const int64_t* __restrict__ row_ptr,
                                                               const int32_t* __restrict__ col,
                                                               const double* __restrict__ val,
@@ -111,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_step_csr_f64(int64_t n, const i
   if (blockIdx.y > 0 && !chunks) return;
   const int64_t first = row < n ? row_ptr[row] : end, stop = row < n ? row_ptr[row + 1] : end;
   auto stage = [&](int64_t c0, int count) {
-#pragma unroll 4
+#pragma unroll AHEAD
     for (int i = tid; i < count; i += kThreads) {
       s_val[place(i)] = __ldcs(val + c0 + i);
       s_col[place(i)] = __ldcs(col + c0 + i);
@@ -190,8 +193,8 @@ __global__ void __launch_bounds__(kThreads, 8) k_step_csr_f64(int64_t n, const i
 // The same step for a matrix of wide rows, where the caller says that it is one: eight lanes a row straight from
 // memory, with all of L1 for the gathers and twice the threads that shared memory leaves above (81 entries a row,
 // us a step, shared rows above / this: 50 thousand rows 27.0 / 15.6, 150 thousand 60.2 / 46.6; 121 entries, 300
-// thousand rows 179.6 / 112.0). The lanes' loop is not unrolled: four entries of a lane at a time lie in other lines than the
-// ones at hand, which its neighbours still read (112.0 us against 157.4).
+// thousand rows 179.6 / 112.0). The lanes' loop is not unrolled: four entries of a lane at a time lie in other lines than
+// the ones at hand, which its neighbours still read (112.0 us against 157.4).
 template <bool FIRST, bool LAST>
 __global__ void __launch_bounds__(256) k_step_csr_wide_f64(int64_t n, const int64_t* __restrict__ row_ptr,
                                                            const int32_t* __restrict__ col,
@@ -218,22 +221,29 @@ __global__ void __launch_bounds__(256) k_step_csr_wide_f64(int64_t n, const int6
   }
 }
 
+enum Kernel { kShort, kStaged, kWide };  // of a call's steps
+
 template <bool FIRST, bool LAST>
-cudaError_t launch_step(bool wide, unsigned split, int64_t n, cudaStream_t st, const int64_t* row_ptr,
+auto kernel_of(Kernel k) {
+  return k == kWide ? k_step_csr_wide_f64<FIRST, LAST>
+                    : k == kShort ? k_step_csr_f64<FIRST, LAST, 8> : k_step_csr_f64<FIRST, LAST, 4>;
+}
+
+template <bool FIRST, bool LAST>
+cudaError_t launch_step(Kernel k, unsigned split, int64_t n, cudaStream_t st, const int64_t* row_ptr,
                         const int32_t* col, const double* val, const double* tau2m, const double* x,
                         const double* prev, double* out, double* acc, const double* alpha, int step) {
   const unsigned groups = static_cast<unsigned>((n + kThreads - 1) / kThreads);
   cudaLaunchConfig_t c{};
-  c.gridDim = wide ? dim3(static_cast<unsigned>((n * kRowLanes + 255) / 256)) : dim3(groups, split);
-  c.blockDim = dim3(wide ? 256 : kThreads);
+  c.gridDim = k == kWide ? dim3(static_cast<unsigned>((n * kRowLanes + 255) / 256)) : dim3(groups, split);
+  c.blockDim = dim3(k == kWide ? 256 : kThreads);
   c.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   c.attrs = at;
   c.numAttrs = FIRST ? 0 : 1;  // the first step follows the caller's own work
-  return cudaLaunchKernelEx(&c, wide ? k_step_csr_wide_f64<FIRST, LAST> : k_step_csr_f64<FIRST, LAST>, n, row_ptr,
-                            col, val, tau2m, x, prev, out, acc, alpha, step);
+  return cudaLaunchKernelEx(&c, kernel_of<FIRST, LAST>(k), n, row_ptr, col, val, tau2m, x, prev, out, acc, alpha, step);
 }
 
 std::mutex g_setup_mu;
@@ -276,11 +286,15 @@ extern "C" kes_status kes_filter_apply_noalloc_sized(int64_t n, int64_t nnz, con
     return KES_ERR_CUDA;
   }
   double* U[2] = {state, state + KES_NOALLOC_MAX_N};
-  const bool wide = n >= kWideRows && nnz / n >= kWideEntries;
+  const int64_t groups = (n + kThreads - 1) / kThreads;
+  const bool narrow = nnz >= 0 && nnz <= 16 * n;  // a row on average fills no more than its share of a chunk
+  const Kernel kernel = n >= kWideRows && nnz / n >= kWideEntries ? kWide
+                        : narrow && groups <= 2 * kBlocks         ? kShort
+                                                                  : kStaged;
   // blocks of a group: not where the rows are known to be short on average (the blocks that leave at once cost a small
   // matrix 4% of a step)
-  unsigned split = nnz >= 0 && nnz <= 16 * n ? 1 : kMaxSplit;
-  while (split > 1 && static_cast<unsigned>((n + kThreads - 1) / kThreads) * split > kBlocks) split /= 2;
+  unsigned split = narrow ? 1 : kMaxSplit;
+  while (split > 1 && groups * split > kBlocks) split /= 2;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   for (int s = 0; s < L; ++s) {
     const bool first = s == 0, last = s == L - 1;
@@ -289,7 +303,7 @@ extern "C" kes_status kes_filter_apply_noalloc_sized(int64_t n, int64_t nnz, con
     double* out = U[s & 1];
     const auto go = first ? (last ? launch_step<true, true> : launch_step<true, false>)
                           : (last ? launch_step<false, true> : launch_step<false, false>);
-    if (go(wide, split, n, st, row_ptr, col, val, tau2m, x, prev, out, r_out, alpha, s) != cudaSuccess) {
+    if (go(kernel, split, n, st, row_ptr, col, val, tau2m, x, prev, out, r_out, alpha, s) != cudaSuccess) {
       cudaGetLastError();
       return KES_ERR_CUDA;
     }
